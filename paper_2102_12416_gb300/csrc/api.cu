@@ -290,6 +290,10 @@ int plan_build(int64_t n_grids, const jacobi_dim3* grids, const jacobi_split* sp
           P->blocks.push_back(B);
         }
     G.block_end = (int64_t)P->blocks.size();
+    for (int64_t b = G.block_begin; b < G.block_end; ++b) {
+      const BlockHost& B = P->blocks[b];
+      G.max_rows = std::max(G.max_rows, (int32_t)((B.extent[1] + 2) * (B.extent[2] + 2)));
+    }
     if (G.block_end > (1ll << 30)) return set_error(JACOBI_EINVAL, "too many blocks");
     P->n_points += d.nx * d.ny * d.nz;
     P->grids.push_back(G);
@@ -902,23 +906,12 @@ int residual_only(jacobi_t* h, cudaStream_t s) {
   return JACOBI_OK;
 }
 
-// |b|^2 and the FP64 adder-domain check of every grid (grid < 0) or of one
-// grid (after its state was replaced).
-int compute_bnorm(jacobi_t* h, cudaStream_t s, int64_t grid) {
+// |b|^2 of every grid from its slots; new_state also publishes the domain
+// flags that the initial-state kernel gathered.
+int compute_bnorm(jacobi_t* h, cudaStream_t s, bool new_state) {
   StepLaunch a = step_args(h, h->iter, true);
-  int32_t b0 = 0, nb = (int32_t)h->plan.blocks.size(), g0 = 0, ng = (int32_t)h->plan.grids.size();
-  if (grid >= 0) {
-    const GridHost& G = h->plan.grids[grid];
-    a.items += G.item_begin;
-    a.n_items = (int32_t)(G.item_end - G.item_begin);
-    b0 = (int32_t)G.block_begin;
-    nb = (int32_t)(G.block_end - G.block_begin);
-    g0 = (int32_t)grid;
-    ng = 1;
-  }
-  JGB_CUDA(launch_emu_check(h->d_blocks + b0, nb, h->d_grids, h->d_norms, h->d_gids + g0, ng, h->iter, h->plan.dtype, s));
   JGB_CUDA(launch_bnorm(a, s));
-  JGB_CUDA(launch_reduce(h->d_grids, h->d_norms, h->d_gids + g0, ng, h->d_partials, 1, s));
+  JGB_CUDA(launch_reduce(h->d_grids, h->d_norms, h->d_gids, (int32_t)h->plan.grids.size(), h->d_partials, new_state ? 1 : 2, s));
   return JACOBI_OK;
 }
 
@@ -998,7 +991,7 @@ int apply_shape(jacobi_t* h, int64_t zchunk, int32_t cw_cap, cudaStream_t s) {
   }
   if (128 + h->stages * (int64_t)P.max_stage > kMaxStepSmem) h->stages = 3;
   h->tables_dirty = true;
-  rc = compute_bnorm(h, s, -1);
+  rc = compute_bnorm(h, s, false);  // the state, and so its domain flag, is the same
   if (rc) return rc;
   return refresh_active(h, s);
 }
@@ -1168,9 +1161,11 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
   if (e != cudaSuccess) return fail(set_error(JACOBI_ECUDA, "workspace clear failed: %s", cudaGetErrorString(e)));
   rc = upload_tables(h, s);
   if (rc) return fail(rc);
-  e = launch_init(h->d_blocks, h->d_geom, (int32_t)P.blocks.size(), h->d_inits, P.dtype, s);
+  int32_t max_rows = 0;
+  for (const GridHost& G : P.grids) max_rows = std::max(max_rows, G.max_rows);
+  e = launch_init(h->d_blocks, h->d_geom, (int32_t)P.blocks.size(), max_rows, h->d_inits, h->d_norms, P.dtype, s);
   if (e != cudaSuccess) return fail(set_error(JACOBI_ECUDA, "init launch failed: %s", cudaGetErrorString(e)));
-  rc = compute_bnorm(h, s, -1);
+  rc = compute_bnorm(h, s, true);
   if (rc) return fail(rc);
   rc = refresh_active(h, s);
   if (rc) return fail(rc);
@@ -1603,11 +1598,12 @@ int jacobi_set_state(jacobi_t* h, int64_t grid, const void* src, int32_t src_on_
     dsrc = tmp;
   }
   const int parity = (int)(grid_local_iter(h, grid) & 1);
-  cudaError_t e = launch_scatter(h->d_blocks, h->d_geom, (int32_t)G.block_begin, (int32_t)(G.block_end - G.block_begin),
-                                 dsrc, G.dims.nx, G.dims.ny, G.dims.nz, parity, h->plan.dtype, s);
+  cudaError_t e = launch_scatter(h->d_blocks, h->d_geom, (int32_t)G.block_begin, (int32_t)(G.block_end - G.block_begin), G.max_rows,
+                                 dsrc, G.dims.nx, G.dims.ny, parity, h->d_items + G.item_begin,
+                                 (int32_t)(G.item_end - G.item_begin), h->d_partials, h->d_norms, h->plan.dtype, s);
+  if (e == cudaSuccess) e = launch_reduce(h->d_grids, h->d_norms, h->d_gids + grid, 1, h->d_partials, 1, s);
   int rc = JACOBI_OK;
   if (e != cudaSuccess) rc = set_error(JACOBI_ECUDA, "scatter failed: %s", cudaGetErrorString(e));
-  if (!rc) rc = compute_bnorm(h, s, grid);
   if (!rc && !src_on_device) {
     // the caller may reuse its host buffer as soon as the call returns
     cudaError_t e2 = cudaStreamSynchronize(s);
@@ -1636,8 +1632,8 @@ int jacobi_copy_out(jacobi_t* h, int64_t grid, void* dst, int32_t dst_on_device,
   if (layout == JACOBI_LAYOUT_PADDED) e = cudaMemsetAsync(ddst, 0, n, s);
   const int parity = (int)(grid_local_iter(h, grid) & 1);
   if (e == cudaSuccess)
-    e = launch_gather(h->d_blocks, h->d_geom, (int32_t)G.block_begin, (int32_t)(G.block_end - G.block_begin), ddst,
-                      G.dims.nx, G.dims.ny, G.dims.nz, parity, layout == JACOBI_LAYOUT_PADDED, h->plan.dtype, s);
+    e = launch_gather(h->d_blocks, h->d_geom, (int32_t)G.block_begin, (int32_t)(G.block_end - G.block_begin), G.max_rows, ddst,
+                      G.dims.nx, G.dims.ny, parity, layout == JACOBI_LAYOUT_PADDED, h->plan.dtype, s);
   if (e == cudaSuccess && tmp) e = cudaMemcpyAsync(dst, tmp, n, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && tmp) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) rc = set_error(JACOBI_ECUDA, "copy_out failed: %s", cudaGetErrorString(e));

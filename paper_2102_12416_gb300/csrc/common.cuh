@@ -75,7 +75,7 @@ struct GridNorm {
   double r_norm;        // sqrt(r_norm2)
   double rel;           // r_norm / |b| (r_norm when |b| == 0)
   uint32_t emu_bad;     // the state has a value outside dadd_nn's domain (widened, for FP32)
-  uint32_t pad_;
+  uint32_t emu_acc;     // the same, gathered while a state is being installed
 };
 
 // Tile shape of the table-driven kernels: 32 x 8 threads, each thread walks z.

@@ -42,195 +42,359 @@ __device__ __forceinline__ int64_t face_elems(const BlockDev& B, int f) {
   return (int64_t)B.ry * B.rx;
 }
 
-// Global padded grid coordinates of slot entry e of face f of block (B, G);
-// false for a padding entry.
-__device__ __forceinline__ bool face_coords(const BlockDev& B, const BlockGeom& G, int f, int64_t e,
-                                            int64_t& gi, int64_t& gj, int64_t& gk) {
-  const int nx = B.nx, ny = B.ny, nz = B.nz;
-  if (f == XM || f == XP) {
-    const int64_t k = e / B.ry, j = e % B.ry;
-    gi = G.ox + (f == XM ? 0 : nx + 1);
-    gj = G.oy + 1 + j;
-    gk = G.oz + 1 + k;
-    return j < ny;
-  }
-  if (f == YM || f == YP) {
-    const int64_t k = e / B.rx, i = e % B.rx;
-    gi = G.ox + 1 + i;
-    gj = G.oy + (f == YM ? 0 : ny + 1);
-    gk = G.oz + 1 + k;
-    return i < nx;
-  }
-  const int64_t j = e / B.rx, i = e % B.rx;
-  gi = G.ox + 1 + i;
-  gj = G.oy + 1 + j;
-  gk = G.oz + (f == ZM ? 0 : nz + 1);
-  return i < nx && j < ny;
-}
-
 // Offset of interior point (i, j, k) in the block's padded storage.
 __device__ __forceinline__ int64_t cell(const BlockDev& B, int64_t i, int64_t j, int64_t k) {
   return k * B.plane_pitch + j * B.rx + i;
 }
 
-// Calls f(i, j, k) for every interior point of B: the CTA's warps take the
-// rows (j, k) in turn, the lanes walk a row (coalesced; one division per row).
-template <typename F>
-__device__ __forceinline__ void for_interior(const BlockDev& B, F f) {
-  const int nx = B.nx, ny = B.ny, rows = B.ny * B.nz;
-  const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  for (int row = threadIdx.x >> 5; row < rows; row += nwarps) {
-    const int k = row / ny, j = row - k * ny;
-    for (int i = lane; i < nx; i += 32) f(i, j, k);
+// ---------------------------------------------------------------------------
+// Whole-state kernels: initial state, scatter from a padded array, gather.
+//
+// Each of them is a pass over memory, so what counts is loads in flight.  A
+// block is walked as *extended rows* (j, k), j in [-1, ny], k in [-1, nz]: a
+// row of the interior, or one of a y or z receive slot (j or k outside), all
+// nx elements long with pitch rx, so interior and slots take the same code; the
+// two x ghosts of an interior row are read beside it.  A block's rows are
+// split over nsub CTAs (state_split), a warp takes 32 / LPR rows at a time (LPR
+// lanes per row, 32 unless the block is narrower), and each lane keeps 4 rows x
+// 2 elements in flight.  With one CTA per block (before) a small grid left most
+// of the chip idle, and a batch paid that once per grid.  jacobi_set_state (with
+// its |b| and domain check) and jacobi_copy_out on the device, before -> now:
+// 64^3 FP64 in 32^3 blocks 130 -> 20 and 51 -> 13 us; 512^3 FP64 in 64^3 blocks
+// 2.69 -> 0.50 and 0.66 -> 0.36 ms; 768^3 FP32 7.8 -> 1.25 and 1.28 -> 0.99 ms; 256
+// FP32 grids of 16..192 set and read back 66 -> 9 ms.
+// ---------------------------------------------------------------------------
+struct RowWalk {
+  int lo, ey, r, r1, step, j, k, sj, sk, x, lpr;
+};
+
+// Rows of this CTA's share; lo = 1 walks the extended rows, 0 the interior only.
+__device__ __forceinline__ RowWalk row_walk(const BlockDev& B, int lo, int sub, int nsub) {
+  RowWalk W;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  W.lo = lo;
+  W.ey = B.ny + 2 * lo;
+  const int rows = W.ey * (B.nz + 2 * lo);
+  int sh = 5;
+  while (sh > 0 && (1 << (sh - 1)) >= B.nx) --sh;  // lanes per row: the power of two >= nx, at most 32
+  W.lpr = 1 << sh;
+  W.x = lane & (W.lpr - 1);
+  const int rpw = 32 >> sh;
+  W.step = nwarps * rpw;
+  W.r = (int)((int64_t)rows * sub / nsub) + warp * rpw + (lane >> sh);
+  W.r1 = (int)((int64_t)rows * (sub + 1) / nsub);
+  W.j = W.r % W.ey;
+  W.k = W.r / W.ey;
+  W.sj = W.step % W.ey;
+  W.sk = W.step / W.ey;
+  return W;
+}
+__device__ __forceinline__ void row_next(RowWalk& W) {
+  W.r += W.step;
+  W.j += W.sj;
+  W.k += W.sk;
+  if (W.j >= W.ey) {
+    W.j -= W.ey;
+    W.k += 1;
   }
 }
 
+// Storage of extended row (j, k) at parity p; null where both are outside.
 template <typename T>
-__global__ void k_init_interior(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
-                                const InitDev* __restrict__ inits) {
-  const BlockDev& B = blocks[blockIdx.x];
+__device__ __forceinline__ T* ext_row(const BlockDev& B, int p, int j, int k) {
+  const bool jo = j < 0 || j >= B.ny, ko = k < 0 || k >= B.nz;
+  if (jo && ko) return nullptr;
+  if (ko) return (T*)B.recv[k < 0 ? ZM : ZP][p] + (int64_t)j * B.rx;
+  if (jo) return (T*)B.recv[j < 0 ? YM : YP][p] + (int64_t)k * B.rx;
+  return (T*)B.u[p] + (int64_t)k * B.plane_pitch + (int64_t)j * B.rx;
+}
+
+// Outside the domain of the integer-pipe adder: sign set, or an exponent field
+// that is too large (FP64) or that of infinities and NaNs (FP32, widened).
+__device__ __forceinline__ bool emu_outside(double v) { return (uint32_t)__double2hiint(v) >= kEmuHiLimit; }
+__device__ __forceinline__ bool emu_outside(float v) { return __float_as_uint(v) >= 0x7F800000u; }
+
+// A grid whose state holds a value outside that domain is flagged: the step
+// kernels then keep its FP64 sums (the FP64 stencil's, and the FP32 residual's
+// of widened values) on the FP64 pipe.  By the discrete maximum principle
+// Jacobi iterates stay within the range of the boundary and initial data, so a
+// state that passes keeps passing.  The kernels that install a state gather the
+// flag in emu_acc; the |b| reduction that follows them publishes it as emu_bad
+// and clears it for the next state.
+__device__ __forceinline__ void emu_flag(bool bad, GridNorm* norms, int grid) {
+  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&norms[grid].emu_acc, 1u);
+}
+
+__device__ __forceinline__ void block_to_shared(BlockDev& d, const BlockDev* s) {
+  for (int q = threadIdx.x; q < (int)(sizeof(BlockDev) / 4); q += blockDim.x) ((uint32_t*)&d)[q] = ((const uint32_t*)s)[q];
+  __syncthreads();
+}
+
+// |b|^2 partial of one work item: the residual expression with every interior
+// value 0, so only points beside a Dirichlet face contribute and only those are
+// visited, each once: the item's z-face planes, the y-face rows of its other
+// planes, the x-face columns of the other rows.  `ghost(f, i, j, k)` is the
+// boundary value across face f of point (i, j, k).  (Visiting every point, as
+// before: 1.5 ms at 512^3 FP64, 5.2 ms at 768^3 FP32.)  The ranges are written
+// with 0/1 flags on purpose: as max() of the 16-bit item fields, ptxas 13.0
+// gave empty ranges at -O1 and above (and right ones at -O0).
+template <typename G>
+__device__ __forceinline__ void bnorm_add(double& acc, const BlockDev& B, const G& ghost, int i, int j, int k) {
+  double v[6] = {0, 0, 0, 0, 0, 0};
+  if (i == 0 && B.nbr[XM] < 0) v[0] = ghost(XM, i, j, k);
+  if (i == B.nx - 1 && B.nbr[XP] < 0) v[1] = ghost(XP, i, j, k);
+  if (j == 0 && B.nbr[YM] < 0) v[2] = ghost(YM, i, j, k);
+  if (j == B.ny - 1 && B.nbr[YP] < 0) v[3] = ghost(YP, i, j, k);
+  if (k == 0 && B.nbr[ZM] < 0) v[4] = ghost(ZM, i, j, k);
+  if (k == B.nz - 1 && B.nbr[ZP] < 0) v[5] = ghost(ZP, i, j, k);
+  const double sb = __dadd_rn(__dadd_rn(__dadd_rn(v[0], v[1]), __dadd_rn(v[2], v[3])), __dadd_rn(v[4], v[5]));
+  acc = fma(sb, sb, acc);
+}
+template <typename G>
+__device__ __forceinline__ double bnorm_item(const BlockDev& B, const WorkItem& w, const G& ghost) {
+  const int nx = B.nx, ny = B.ny, nz = B.nz, tid = threadIdx.x;
+  const int za = w.z0, zb = w.z1;
+  const int xa = w.x0 >= 0 ? w.x0 : 0, ya = w.x0 >= 0 ? w.y0 : w.ya;
+  const int xb = w.x0 >= 0 ? min(w.x0 + TX, nx) : nx, yb = min(w.x0 >= 0 ? w.y0 + TY : (int)w.yb, ny);
+  double acc = 0.0;
+  // Planes (rows, columns) of the item on its low and high Dirichlet faces: 0
+  // or 1 each (a one-point extent with both faces counts as low).  Planes
+  // [ka, kb), rows [ja, jb) and columns [ia, ib) are away from them.
+  const int zlo = (za == 0 && B.nbr[ZM] < 0) ? 1 : 0, zhi = (zb == nz && B.nbr[ZP] < 0 && zb - za > zlo) ? 1 : 0;
+  const int ylo = (ya == 0 && B.nbr[YM] < 0) ? 1 : 0, yhi = (yb == ny && B.nbr[YP] < 0 && yb - ya > ylo) ? 1 : 0;
+  const int xlo = (xa == 0 && B.nbr[XM] < 0) ? 1 : 0, xhi = (xb == nx && B.nbr[XP] < 0 && xb - xa > xlo) ? 1 : 0;
+  const int ka = za + zlo, kb = zb - zhi, ja = ya + ylo, jb = yb - yhi, ib = xb - xhi;
+  const int nw = xb - xa, nh = yb - ya, nd = kb - ka, nr = jb - ja;
+  // One loop over the points of all three groups: the first e of each group's
+  // plane (row, column) are those before the inner range, the others after it.
+  const int ez = nw * nh * (zlo + zhi), ey = ez + nw * nd * (ylo + yhi), ex = ey + nr * nd * (xlo + xhi);
+  for (int e = tid; e < ex; e += kThreads) {
+    int i, j, k;
+    if (e < ez) {
+      const int n = nw * nh, t = e / n, q = e - t * n;
+      k = t < zlo ? za + t : kb + t - zlo;
+      j = ya + q / nw;
+      i = xa + q % nw;
+    } else if (e < ey) {
+      const int n = nw * nd, t = (e - ez) / n, q = (e - ez) - t * n;
+      j = t < ylo ? ya + t : jb + t - ylo;
+      k = ka + q / nw;
+      i = xa + q % nw;
+    } else {
+      const int n = nr * nd, t = (e - ey) / n, q = (e - ey) - t * n;
+      i = t < xlo ? xa + t : ib + t - xlo;
+      k = ka + q / nr;
+      j = ja + q % nr;
+    }
+    bnorm_add(acc, B, ghost, i, j, k);
+  }
+  return acc;
+}
+
+// Boundary values from the receive slots of parity p, or from a padded array
+// (base: the block's first interior point).
+template <typename T>
+struct SlotGhost {
+  const BlockDev* B;
+  int p;
+  __device__ __forceinline__ double operator()(int f, int i, int j, int k) const {
+    const int64_t e = f < YM ? (int64_t)k * B->ry + j : f < ZM ? (int64_t)k * B->rx + i : (int64_t)j * B->rx + i;
+    return (double)((const T*)B->recv[f][p])[e];
+  }
+};
+template <typename T>
+struct ArrayGhost {
+  const T* base;
+  int64_t px, pp;  // row and plane pitch
+  __device__ __forceinline__ double operator()(int f, int i, int j, int k) const {
+    const int64_t d = f < YM ? 1 : f < ZM ? px : pp;
+    return (double)base[(int64_t)k * pp + (int64_t)j * px + i + ((f & 1) ? d : -d)];
+  }
+};
+
+// Initial state (interior and slots at parity 0) with its domain check.  The
+// workspace is zero before this kernel, so a zero interior is not written.
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_init(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
+                                                   const InitDev* __restrict__ inits, GridNorm* norms) {
+  __shared__ BlockDev B;
+  block_to_shared(B, blocks + blockIdx.x);
   const BlockGeom G = geom[blockIdx.x];
   const InitDev I = inits[G.grid];
-  T* U = (T*)B.u[0];
-  // a flat walk: for a zero interior this is a pure store stream, which the
-  // row-wise walk issued ~3x slower
-  const int64_t nx = B.nx, ny = B.ny, n = nx * ny * B.nz, pitch = B.plane_pitch, rx = B.rx;
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    const int64_t i = e % nx, j = (e / nx) % ny, k = e / (nx * ny);
-    U[k * pitch + j * rx + i] = to_state<T>(init_value(I, G.ox + 1 + i, G.oy + 1 + j, G.oz + 1 + k));
+  bool bad = false;
+  auto value = [&](int i, int j, int k) {
+    const T v = to_state<T>(init_value(I, G.ox + 1 + i, G.oy + 1 + j, G.oz + 1 + k));
+    bad |= emu_outside(v);
+    return v;
+  };
+  for (RowWalk W = row_walk(B, 1, blockIdx.y, gridDim.y); W.r < W.r1; row_next(W)) {
+    const int j = W.j - 1, k = W.k - 1;
+    T* d = ext_row<T>(B, 0, j, k);
+    if (!d) continue;
+    const bool inside = j >= 0 && j < B.ny && k >= 0 && k < B.nz;
+    if (!inside || I.interior != 0)
+      for (int i = W.x; i < B.nx; i += W.lpr) d[i] = value(i, j, k);
   }
+  // x slots: lanes along y, so that a warp's FP64 divisions serve 32 values
+  const int64_t n = (int64_t)B.ny * B.nz;
+  const int64_t e1 = 2 * n * (blockIdx.y + 1) / gridDim.y;
+  for (int64_t e = 2 * n * blockIdx.y / gridDim.y + threadIdx.x; e < e1; e += kThreads) {
+    const int q = (int)(e < n ? e : e - n), k = q / B.ny, j = q - k * B.ny;
+    ((T*)B.recv[e < n ? XM : XP][0])[(int64_t)k * B.ry + j] = value(e < n ? -1 : B.nx, j, k);
+  }
+  emu_flag(bad, norms, G.grid);
 }
 
+// CTAs [0, nb * nsub) install a padded array of one grid into its blocks
+// (parity p state and slots) and check its domain; the CTAs after them take one
+// work item each and write its |b|^2 partial, straight from the array.
 template <typename T>
-__global__ void k_init_slots(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
-                             const InitDev* __restrict__ inits) {
-  const BlockDev& B = blocks[blockIdx.x];
-  const BlockGeom G = geom[blockIdx.x];
-  const InitDev I = inits[G.grid];
-  const int f = blockIdx.y;
-  T* S = (T*)B.recv[f][0];
-  const int64_t n = face_elems(B, f);
-  for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-    int64_t gi, gj, gk;
-    if (face_coords(B, G, f, e, gi, gj, gk)) S[e] = to_state<T>(init_value(I, gi, gj, gk));
-  }
-}
-
-template <typename T>
-__global__ void k_scatter(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom, int32_t b0,
-                          const T* __restrict__ src, int64_t NX, int64_t NY, int parity) {
-  const int b = b0 + blockIdx.x;
-  const BlockDev& B = blocks[b];
-  const BlockGeom G = geom[b];
+__global__ void __launch_bounds__(kThreads, 4) k_scatter(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
+                                                      int32_t b0, int32_t nb, int32_t nsub, const T* __restrict__ src, int64_t NX,
+                                                      int64_t NY, int parity, const WorkItem* __restrict__ items, double* partials,
+                                                      GridNorm* norms) {
+  __shared__ BlockDev B;
   const int64_t px = NX + 2, py = NY + 2;
-  if (blockIdx.y == 0) {
-    T* U = (T*)B.u[parity];
-    const int64_t pitch = B.plane_pitch, rx = B.rx;
-    for_interior(B, [=](int i, int j, int k) {
-      U[k * pitch + j * rx + i] = src[((G.oz + 1 + k) * py + (G.oy + 1 + j)) * px + (G.ox + 1 + i)];
-    });
-  } else {
-    const int f = blockIdx.y - 1;
-    T* S = (T*)B.recv[f][parity];
-    const int64_t n = face_elems(B, f);
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-      int64_t gi, gj, gk;
-      if (face_coords(B, G, f, e, gi, gj, gk)) S[e] = src[(gk * py + gj) * px + gi];
-    }
+  if ((int)blockIdx.x >= nb * nsub) {
+    const WorkItem w = items[blockIdx.x - nb * nsub];
+    block_to_shared(B, blocks + w.block);
+    const BlockGeom G = geom[w.block];
+    const T* base = src + ((int64_t)(G.oz + 1) * py + (G.oy + 1)) * px + (G.ox + 1);
+    const double acc = bnorm_item(B, w, ArrayGhost<T>{base, px, px * py});
+    __shared__ double red[kThreads / 32];
+    const double s = block_sum<kThreads>(acc, red);
+    if (threadIdx.x == 0) partials[w.slot] = s;
+    return;
   }
-}
-
-template <typename T>
-__global__ void k_gather(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom, int32_t b0,
-                         T* __restrict__ dst, int64_t NX, int64_t NY, int parity, int padded) {
-  const int b = b0 + blockIdx.x;
-  const BlockDev& B = blocks[b];
+  const int b = b0 + blockIdx.x / nsub;
+  block_to_shared(B, blocks + b);
   const BlockGeom G = geom[b];
-  const int64_t off = padded ? 1 : 0;
-  const int64_t px = NX + 2 * off, py = NY + 2 * off;
-  if (blockIdx.y == 0) {
-    const T* U = (const T*)B.u[parity];
-    const int64_t pitch = B.plane_pitch, rx = B.rx;
-    for_interior(B, [=](int i, int j, int k) {
-      dst[((G.oz + off + k) * py + (G.oy + off + j)) * px + (G.ox + off + i)] = U[k * pitch + j * rx + i];
-    });
-  } else if (padded) {
-    const int f = blockIdx.y - 1;
-    if (B.nbr[f] >= 0) return;  // only Dirichlet faces lie on the padded boundary
-    const T* S = (const T*)B.recv[f][parity];
-    const int64_t n = face_elems(B, f);
-    for (int64_t e = threadIdx.x; e < n; e += blockDim.x) {
-      int64_t gi, gj, gk;
-      if (face_coords(B, G, f, e, gi, gj, gk)) dst[(gk * py + gj) * px + gi] = S[e];
+  const T* __restrict__ base = src + ((int64_t)(G.oz + 1) * py + (G.oy + 1)) * px + (G.ox + 1);
+  const int nx = B.nx;
+  bool bad = false;
+  RowWalk W = row_walk(B, 1, blockIdx.x % nsub, nsub);
+  while (W.r < W.r1) {
+    constexpr int U = 4;
+    const T* s[U];
+    T* d[U];
+    int ge[U];  // an interior row's entry in the x slots, else -1
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = W.j - 1, k = W.k - 1;
+      d[u] = W.r < W.r1 ? ext_row<T>(B, parity, j, k) : nullptr;
+      s[u] = base + ((int64_t)k * py + j) * px;
+      const bool inside = d[u] && j >= 0 && j < B.ny && k >= 0 && k < B.nz;
+      ge[u] = inside ? k * B.ry + j : -1;
+      row_next(W);
+    }
+    T g[U];
+    const int gi = W.x == 0 ? -1 : nx;
+    if (W.x < 2) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (ge[u] >= 0) g[u] = s[u][gi];
+    }
+    for (int i = W.x; i < nx; i += 2 * W.lpr) {
+      T v[U][2];
+      const bool two = i + W.lpr < nx;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (d[u]) {
+          v[u][0] = s[u][i];
+          if (two) v[u][1] = s[u][i + W.lpr];
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (d[u]) {
+          d[u][i] = v[u][0];
+          bad |= emu_outside(v[u][0]);
+          if (two) {
+            d[u][i + W.lpr] = v[u][1];
+            bad |= emu_outside(v[u][1]);
+          }
+        }
+    }
+    if (W.x < 2) {
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (ge[u] >= 0) {
+          ((T*)B.recv[W.x == 0 ? XM : XP][parity])[ge[u]] = g[u];
+          bad |= emu_outside(g[u]);
+          if (W.lpr == 1) {  // one-point rows: this lane takes both ghosts
+            const T o = s[u][nx];
+            ((T*)B.recv[XP][parity])[ge[u]] = o;
+            bad |= emu_outside(o);
+          }
+        }
+    }
+  }
+  emu_flag(bad, norms, G.grid);
+}
+
+// Current iterate (parity p) back to an array of the whole grid: the interior,
+// or (padded) with the Dirichlet faces around it.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 4) k_gather(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
+                                                     int32_t b0, int32_t nsub, T* __restrict__ dst, int64_t NX, int64_t NY, int parity,
+                                                     int padded) {
+  __shared__ BlockDev B;
+  const int b = b0 + blockIdx.x / nsub;
+  block_to_shared(B, blocks + b);
+  const BlockGeom G = geom[b];
+  const int64_t px = NX + 2 * padded, py = NY + 2 * padded;
+  T* __restrict__ base = dst + ((int64_t)(G.oz + padded) * py + (G.oy + padded)) * px + (G.ox + padded);
+  const int nx = B.nx;
+  RowWalk W = row_walk(B, padded, blockIdx.x % nsub, nsub);
+  while (W.r < W.r1) {
+    constexpr int U = 4;
+    const T* s[U];
+    T* d[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = W.j - padded, k = W.k - padded;
+      bool take = W.r < W.r1;
+      if (padded) {  // only Dirichlet faces lie on the padded boundary
+        if (j < 0) take = take && B.nbr[YM] < 0;
+        if (j >= B.ny) take = take && B.nbr[YP] < 0;
+        if (k < 0) take = take && B.nbr[ZM] < 0;
+        if (k >= B.nz) take = take && B.nbr[ZP] < 0;
+      }
+      s[u] = take ? ext_row<T>(B, parity, j, k) : nullptr;
+      d[u] = base + ((int64_t)k * py + j) * px;
+      if (padded && s[u] && j >= 0 && j < B.ny && k >= 0 && k < B.nz)
+        for (int g = W.x; g < 2; g += W.lpr)
+          if (B.nbr[g ? XP : XM] < 0) d[u][g ? nx : -1] = ((const T*)B.recv[g ? XP : XM][parity])[(int64_t)k * B.ry + j];
+      row_next(W);
+    }
+    for (int i = W.x; i < nx; i += 2 * W.lpr) {
+      T v[U][2];
+      const bool two = i + W.lpr < nx;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (s[u]) {
+          v[u][0] = s[u][i];
+          if (two) v[u][1] = s[u][i + W.lpr];
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (s[u]) {
+          d[u][i] = v[u][0];
+          if (two) d[u][i + W.lpr] = v[u][1];
+        }
     }
   }
 }
 
-// |b|^2 partials: the residual expression with every interior value set to 0,
-// so only Dirichlet ghosts contribute.  A work item is either one TX x TY tile
-// (x0 >= 0) or the row window [ya, yb) of its block's planes over [z0, z1)
-// (x0 < 0; a plane may be split into several windows, each its own item).
+// |b|^2 partials of work items from the receive slots.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) k_bnorm(StepLaunch a) {
   const WorkItem w = a.items[blockIdx.x];
   const BlockDev& B = a.blocks[w.block];
   const int p = (int)((a.it - a.grids[B.grid].start_iter) & 1);
-  const int nx = B.nx, ny = B.ny, nz = B.nz, rx = B.rx, ry = B.ry;
-  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-  const int xa = w.x0 >= 0 ? w.x0 : 0, ya = w.x0 >= 0 ? w.y0 : w.ya;
-  const int xb = w.x0 >= 0 ? w.x0 + TX : nx, yb = min(w.x0 >= 0 ? w.y0 + TY : (int)w.yb, ny);
-  double acc = 0.0;
-  for (int y0 = ya; y0 < yb; y0 += TY)
-    for (int x0 = xa; x0 < xb; x0 += TX) {
-      const int i = x0 + tx, j = y0 + ty;
-      if (i >= nx || j >= yb) continue;
-      for (int k = w.z0; k < w.z1; ++k) {
-        double v[6] = {0, 0, 0, 0, 0, 0};
-        if (i == 0 && B.nbr[XM] < 0) v[0] = (double)((const T*)B.recv[XM][p])[(int64_t)k * ry + j];
-        if (i == nx - 1 && B.nbr[XP] < 0) v[1] = (double)((const T*)B.recv[XP][p])[(int64_t)k * ry + j];
-        if (j == 0 && B.nbr[YM] < 0) v[2] = (double)((const T*)B.recv[YM][p])[(int64_t)k * rx + i];
-        if (j == ny - 1 && B.nbr[YP] < 0) v[3] = (double)((const T*)B.recv[YP][p])[(int64_t)k * rx + i];
-        if (k == 0 && B.nbr[ZM] < 0) v[4] = (double)((const T*)B.recv[ZM][p])[(int64_t)j * rx + i];
-        if (k == nz - 1 && B.nbr[ZP] < 0) v[5] = (double)((const T*)B.recv[ZP][p])[(int64_t)j * rx + i];
-        const double sb =
-            __dadd_rn(__dadd_rn(__dadd_rn(v[0], v[1]), __dadd_rn(v[2], v[3])), __dadd_rn(v[4], v[5]));
-        acc = fma(sb, sb, acc);
-      }
-    }
+  const double acc = bnorm_item(B, w, SlotGhost<T>{&B, p});
   __shared__ double red[kThreads / 32];
   const double s = block_sum<kThreads>(acc, red);
   if (threadIdx.x == 0) a.partials[w.slot] = s;
-}
-
-// Flag every grid whose current state (interior at its parity and all six
-// receive slots) holds a value outside the domain of the integer-pipe adder
-// dadd_nn; the step kernels then keep that grid's FP64 sums (the FP64
-// stencil's, and the FP32 residual's of widened values) on the FP64 pipe.  By the
-// discrete maximum principle Jacobi iterates stay within the range of the
-// boundary and initial data, so a state that passes keeps passing.
-template <typename T>
-__global__ void k_emu_check(const BlockDev* __restrict__ blocks, const GridDev* grids, GridNorm* norms, int64_t it) {
-  // FP64: the high word (sign clear, exponent below 2040); FP32: the whole
-  // word (sign clear, finite: widened, such a value is inside the domain)
-  constexpr int W = sizeof(T) / 4;
-  constexpr uint32_t kLimit = sizeof(T) == 8 ? kEmuHiLimit : 0x7F800000u;
-  const BlockDev& B = blocks[blockIdx.x];
-  const int p = (int)((it - grids[B.grid].start_iter) & 1);
-  const uint32_t* U = (const uint32_t*)B.u[p];
-  bool bad = false;
-  const int64_t pitch = B.plane_pitch, rx = B.rx;
-  for_interior(B, [&](int i, int j, int k) { bad |= U[W * (k * pitch + j * rx + i) + W - 1] >= kLimit; });
-  for (int f = 0; f < 6; ++f) {
-    const uint32_t* S = (const uint32_t*)B.recv[f][p];
-    const int64_t m = face_elems(B, f);
-    for (int64_t e = threadIdx.x; e < m; e += blockDim.x) bad |= S[W * e + W - 1] >= kLimit;
-  }
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&norms[B.grid].emu_bad, 1u);
-}
-
-__global__ void k_emu_reset(GridNorm* norms, const int32_t* grid_ids, int n) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n) norms[grid_ids[q]].emu_bad = 0u;
 }
 
 // Self-test of the integer-pipe adder: out[i] = dadd_nn(a[i], b[i]).
@@ -287,16 +451,19 @@ __global__ void k_pipe_rate(double* out, int iters) {
   out[blockIdx.x * blockDim.x + threadIdx.x] = s;
 }
 
-// One warp per grid: lane l sums slots item_begin + l, + l + 32, ... in order,
-// then a fixed butterfly combines the lanes.
-__global__ void k_reduce(const GridDev* grids, GridNorm* norms, const int32_t* grid_ids, const double* partials,
-                         int which) {
+// One CTA per grid: thread t sums slots item_begin + t, + t + 256, ... in order,
+// then a fixed tree combines the threads (one warp per grid took 16 us for
+// the 4096 partials of a 512^3 grid).  which = 0: the residual; 1: |b| of a
+// newly installed state, which also publishes its domain flag; 2: |b| only.
+__global__ void __launch_bounds__(kThreads) k_reduce(const GridDev* grids, GridNorm* norms, const int32_t* grid_ids,
+                                                     const double* partials, int which) {
   const int g = grid_ids[blockIdx.x];
   const GridDev G = grids[g];
   GridNorm& N = norms[g];
   double s = 0.0;
-  for (int q = G.item_begin + threadIdx.x; q < G.item_end; q += 32) s += partials[q];
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  for (int q = G.item_begin + threadIdx.x; q < G.item_end; q += kThreads) s += partials[q];
+  __shared__ double red[kThreads / 32];
+  s = block_sum<kThreads>(s, red);
   if (threadIdx.x == 0) {
     if (which == 0) {
       N.r_norm2 = s;
@@ -305,6 +472,10 @@ __global__ void k_reduce(const GridDev* grids, GridNorm* norms, const int32_t* g
       N.rel = b > 0.0 ? N.r_norm / b : N.r_norm;
     } else {
       N.b_norm2 = s;
+      if (which == 1) {
+        N.emu_bad = N.emu_acc;
+        N.emu_acc = 0u;
+      }
     }
   }
 }
@@ -375,7 +546,7 @@ cudaError_t launch_bnorm(const StepLaunch& a, cudaStream_t s) {
 cudaError_t launch_reduce(const GridDev* grids, GridNorm* norms, const int32_t* grid_ids, int32_t n,
                           const double* partials, int which, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_reduce<<<n, 32, 0, s>>>(grids, norms, grid_ids, partials, which);
+  k_reduce<<<n, kThreads, 0, s>>>(grids, norms, grid_ids, partials, which);
   return cudaGetLastError();
 }
 
@@ -394,16 +565,6 @@ cudaError_t launch_copy_faces(const BlockDev* blocks, const int32_t* ids, int32_
   const dim3 grid(n_blocks, 6);
   if (dtype == 0) k_copy_faces<double><<<grid, 256, 0, s>>>(blocks, ids, staging, grids, it);
   else k_copy_faces<float><<<grid, 256, 0, s>>>(blocks, ids, staging, grids, it);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_emu_check(const BlockDev* blocks, int32_t n_blocks, const GridDev* grids, GridNorm* norms,
-                             const int32_t* grid_ids, int32_t n_grids, int64_t it, int dtype, cudaStream_t s) {
-  if (n_grids > 0) k_emu_reset<<<(n_grids + 127) / 128, 128, 0, s>>>(norms, grid_ids, n_grids);
-  if (n_blocks > 0) {
-    if (dtype == 0) k_emu_check<double><<<n_blocks, 256, 0, s>>>(blocks, grids, norms, it);
-    else k_emu_check<float><<<n_blocks, 256, 0, s>>>(blocks, grids, norms, it);
-  }
   return cudaGetLastError();
 }
 
@@ -429,37 +590,46 @@ cudaError_t launch_selftest_div6(unsigned long long* bad, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_init(const BlockDev* blocks, const BlockGeom* geom, int32_t n_blocks, const InitDev* inits,
-                        int32_t dtype, cudaStream_t s) {
+// CTAs per block of the whole-state kernels for blocks of up to max_rows
+// extended rows: 512 rows per CTA on large states (64 rows per warp: several
+// batches of loads each, and enough CTAs for an even tail), down to 32 (one batch)
+// while that leaves fewer than about four CTAs per SM.
+static int state_split(int32_t n_blocks, int32_t max_rows) {
+  const int64_t rows = (int64_t)n_blocks * max_rows;
+  const int64_t per = std::min<int64_t>(512, std::max<int64_t>(32, rows / 608));
+  return (int)std::min<int64_t>(65535, (max_rows + per - 1) / per);
+}
+
+cudaError_t launch_init(const BlockDev* blocks, const BlockGeom* geom, int32_t n_blocks, int32_t max_rows,
+                        const InitDev* inits, GridNorm* norms, int32_t dtype, cudaStream_t s) {
   if (n_blocks <= 0) return cudaSuccess;
-  if (dtype == 0) {
-    k_init_interior<double><<<n_blocks, 256, 0, s>>>(blocks, geom, inits);
-    k_init_slots<double><<<dim3(n_blocks, 6), 256, 0, s>>>(blocks, geom, inits);
-  } else {
-    k_init_interior<float><<<n_blocks, 256, 0, s>>>(blocks, geom, inits);
-    k_init_slots<float><<<dim3(n_blocks, 6), 256, 0, s>>>(blocks, geom, inits);
-  }
+  const dim3 grid(n_blocks, state_split(n_blocks, max_rows));
+  if (dtype == 0) k_init<double><<<grid, kThreads, 0, s>>>(blocks, geom, inits, norms);
+  else k_init<float><<<grid, kThreads, 0, s>>>(blocks, geom, inits, norms);
   return cudaGetLastError();
 }
 
-cudaError_t launch_scatter(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, const void* src,
-                           int64_t NX, int64_t NY, int64_t NZ, int parity, int32_t dtype, cudaStream_t s) {
-  (void)NZ;
+cudaError_t launch_scatter(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, int32_t max_rows,
+                           const void* src, int64_t NX, int64_t NY, int parity, const WorkItem* items, int32_t n_items,
+                           double* partials, GridNorm* norms, int32_t dtype, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
-  const dim3 grid(nb, 7);
-  if (dtype == 0) k_scatter<double><<<grid, 256, 0, s>>>(blocks, geom, b0, (const double*)src, NX, NY, parity);
-  else k_scatter<float><<<grid, 256, 0, s>>>(blocks, geom, b0, (const float*)src, NX, NY, parity);
+  const int nsub = state_split(nb, max_rows);
+  const unsigned grid = (unsigned)((int64_t)nb * nsub + n_items);
+  if (dtype == 0)
+    k_scatter<double><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nb, nsub, (const double*)src, NX, NY, parity, items, partials, norms);
+  else
+    k_scatter<float><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nb, nsub, (const float*)src, NX, NY, parity, items, partials, norms);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, void* dst,
-                          int64_t NX, int64_t NY, int64_t NZ, int parity, int padded, int32_t dtype,
-                          cudaStream_t s) {
-  (void)NZ;
+cudaError_t launch_gather(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, int32_t max_rows, void* dst,
+                          int64_t NX, int64_t NY, int parity, int padded, int32_t dtype, cudaStream_t s) {
   if (nb <= 0) return cudaSuccess;
-  const dim3 grid(nb, 7);
-  if (dtype == 0) k_gather<double><<<grid, 256, 0, s>>>(blocks, geom, b0, (double*)dst, NX, NY, parity, padded);
-  else k_gather<float><<<grid, 256, 0, s>>>(blocks, geom, b0, (float*)dst, NX, NY, parity, padded);
+  const int nsub = state_split(nb, max_rows);
+  const unsigned grid = (unsigned)((int64_t)nb * nsub);
+  const int pad = padded ? 1 : 0;
+  if (dtype == 0) k_gather<double><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nsub, (double*)dst, NX, NY, parity, pad);
+  else k_gather<float><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nsub, (float*)dst, NX, NY, parity, pad);
   return cudaGetLastError();
 }
 

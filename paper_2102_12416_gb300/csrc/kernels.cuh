@@ -110,10 +110,7 @@ struct CopyDesc {
 };
 cudaError_t launch_copy_desc(const CopyDesc* d, int32_t n, cudaStream_t s);
 
-// Domain check of the integer-pipe FP64 adder (sets GridNorm::emu_bad) and
-// its self-test.
-cudaError_t launch_emu_check(const BlockDev* blocks, int32_t n_blocks, const GridDev* grids, GridNorm* norms,
-                             const int32_t* grid_ids, int32_t n_grids, int64_t it, int dtype, cudaStream_t s);
+// Self-tests and pipe-rate probe of the integer-pipe arithmetic.
 cudaError_t launch_selftest_dadd(const double* a, const double* b, int64_t n, double* out, cudaStream_t s);
 cudaError_t launch_selftest_widen(unsigned long long* bad, cudaStream_t s);
 cudaError_t launch_selftest_div6(unsigned long long* bad, cudaStream_t s);
@@ -122,23 +119,27 @@ cudaError_t launch_pipe_rate(bool emu, int blocks, int threads, int iters, doubl
 // |b|^2 partials (interior = 0, only Dirichlet ghosts).
 cudaError_t launch_bnorm(const StepLaunch& a, cudaStream_t s);
 
-// Sum partials per grid in a fixed order.  which = 0: r_norm2, 1: b_norm2.
+// Sum partials per grid in a fixed order.  which = 0: r_norm2; 1: b_norm2 of a
+// newly installed state, publishing its domain flag (emu_acc -> emu_bad); 2:
+// b_norm2 only.
 cudaError_t launch_reduce(const GridDev* grids, GridNorm* norms, const int32_t* grid_ids, int32_t n,
                           const double* partials, int which, cudaStream_t s);
 
 // Initial state: interiors of every block and every receive slot (parity 0
-// for internal faces; the shared buffer for Dirichlet faces).
-cudaError_t launch_init(const BlockDev* blocks, const BlockGeom* geom, int32_t n_blocks,
-                        const InitDev* inits, int32_t dtype, cudaStream_t s);
+// for internal faces; the shared buffer for Dirichlet faces), with the domain
+// check of the integer-pipe adder (emu_acc).  The workspace is zero before.
+// max_rows: most extended rows (ny + 2) * (nz + 2) of a block.
+cudaError_t launch_init(const BlockDev* blocks, const BlockGeom* geom, int32_t n_blocks, int32_t max_rows,
+                        const InitDev* inits, GridNorm* norms, int32_t dtype, cudaStream_t s);
 
 // Scatter a padded device array of one grid into its blocks (parity p buffers
-// and slots); gather the current iterate back (interior or padded layout).
-cudaError_t launch_scatter(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb,
-                           const void* src, int64_t NX, int64_t NY, int64_t NZ, int parity,
-                           int32_t dtype, cudaStream_t s);
-cudaError_t launch_gather(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb,
-                          void* dst, int64_t NX, int64_t NY, int64_t NZ, int parity, int padded,
-                          int32_t dtype, cudaStream_t s);
+// and slots) with the domain check, and the |b|^2 partials of its work items;
+// gather the current iterate back (interior or padded layout).
+cudaError_t launch_scatter(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, int32_t max_rows,
+                           const void* src, int64_t NX, int64_t NY, int parity, const WorkItem* items, int32_t n_items,
+                           double* partials, GridNorm* norms, int32_t dtype, cudaStream_t s);
+cudaError_t launch_gather(const BlockDev* blocks, const BlockGeom* geom, int32_t b0, int32_t nb, int32_t max_rows,
+                          void* dst, int64_t NX, int64_t NY, int parity, int padded, int32_t dtype, cudaStream_t s);
 
 // Persistent path: one cooperative launch runs n_iters iterations.
 struct PersistLaunch {

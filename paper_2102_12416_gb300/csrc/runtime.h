@@ -46,6 +46,7 @@ struct GridHost {
   int64_t counts[3];
   int64_t block_begin, block_end;
   int64_t item_begin, item_end;
+  int32_t max_rows = 0;  // most extended rows (ny + 2) * (nz + 2) of a block
   int64_t start_iter;    // global iteration at which the local count was 0
   int64_t frozen_local;  // local iteration held while inactive
   bool active;

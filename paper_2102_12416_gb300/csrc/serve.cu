@@ -221,8 +221,8 @@ int admit(serve_s* s, int si, const Req& q) {
   ENG_CUDA(cudaMemcpyAsync(s->d_slotdev + si, &sd, sizeof sd, cudaMemcpyHostToDevice, st));
   ENG_CUDA(cudaMemcpyAsync(s->d_rec + si, &rec, sizeof rec, cudaMemcpyHostToDevice, st));
   ENG_CUDA(cudaMemsetAsync(sl.ws, 0, P.bytes, st));  // padding starts at zero
-  ENG_CUDA(launch_init(s->d_blocks + sl.block_base, s->d_geom + sl.block_base, (int32_t)nb, s->d_inits,
-                       s->cfg.dtype, st));
+  ENG_CUDA(launch_init(s->d_blocks + sl.block_base, s->d_geom + sl.block_base, (int32_t)nb, G.max_rows, s->d_inits,
+                       s->d_norms, s->cfg.dtype, st));
   StepLaunch a{};
   a.blocks = s->d_blocks;
   a.items = s->d_slot_items + si * kItemsPerSlot;
@@ -231,8 +231,6 @@ int admit(serve_s* s, int si, const Req& q) {
   a.it = s->it;
   a.partials = s->d_partials;
   a.dtype = s->cfg.dtype;
-  ENG_CUDA(launch_emu_check(s->d_blocks + sl.block_base, (int32_t)nb, s->d_grids, s->d_norms, s->d_ids + si, 1,
-                            s->it, s->cfg.dtype, st));
   ENG_CUDA(launch_bnorm(a, st));
   ENG_CUDA(launch_reduce(s->d_grids, s->d_norms, s->d_ids + si, 1, s->d_partials, 1, st));
   // No synchronisation: a host-to-device cudaMemcpyAsync from pageable memory
@@ -332,8 +330,8 @@ int retire_finished(serve_s* s) {
       const size_t bytes = (size_t)G.dims.nx * G.dims.ny * G.dims.nz * sl.plan.elem;
       void* tmp = nullptr;
       ENG_CUDA(cudaMallocAsync(&tmp, bytes, s->stream));
-      ENG_CUDA(launch_gather(s->d_blocks, s->d_geom, (int32_t)sl.block_base, (int32_t)sl.plan.blocks.size(), tmp,
-                             G.dims.nx, G.dims.ny, G.dims.nz, (int)(R.iters & 1), 0, s->cfg.dtype, s->stream));
+      ENG_CUDA(launch_gather(s->d_blocks, s->d_geom, (int32_t)sl.block_base, (int32_t)sl.plan.blocks.size(), G.max_rows, tmp,
+                             G.dims.nx, G.dims.ny, (int)(R.iters & 1), 0, s->cfg.dtype, s->stream));
       ENG_CUDA(cudaMemcpyAsync(sl.out, tmp, bytes, cudaMemcpyDeviceToHost, s->stream));
       ENG_CUDA(cudaFreeAsync(tmp, s->stream));
       ENG_CUDA(cudaStreamSynchronize(s->stream));
