@@ -265,6 +265,43 @@ __device__ __forceinline__ double widen_f32(float f) {
   return __longlong_as_double((long long)(bits | ((uint64_t)(u >> 31) << 63)));
 }
 
+// Error of the rounded sum t = RN(a + b), exactly (Knuth's TwoSum, which needs
+// no order of a and b; exact unless t overflows, subnormals included).
+__device__ __forceinline__ float two_sum_err(float a, float b, float t) {
+  const float bb = __fsub_rn(t, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(t, bb)), __fsub_rn(b, bb));
+}
+
+// FP64 residual r = s - 6u of a point of an FP32 state as a pair of floats,
+// r = d + e.  The FP64 pipe is 1/64 as fast as the FP32 one, so the sum is not
+// taken in FP64 (8 operations per point with r's square) but in FP32 together
+// with the exact rounding error of each of its five additions, of 6u and of the
+// difference; only the last addition d + e and the square are left to FP64.
+// The error terms are multiples of the smallest neighbour's ulp and at most
+// half an ulp of s: their FP32 sum e is exact while the nonzero neighbours
+// (and u) span up to 2^19, and beyond that off by at most 2^-24 of itself,
+// 2^-46 of s.  Where the FP64 sums are exact too (a span of up to 2^26) r is
+// the same number.  False when an operation overflowed, or on a NaN: the caller
+// then takes the sums in FP64.
+__device__ __forceinline__ bool resid_split(float xm, float xp, float ym, float yp, float zm, float zp, float c, float& d,
+                                            float& e) {
+  const float tx = __fadd_rn(xm, xp), ty = __fadd_rn(ym, yp), tz = __fadd_rn(zm, zp);
+  const float ta = __fadd_rn(tx, ty), s = __fadd_rn(ta, tz);
+  const float ph = __fmul_rn(6.0f, c), pl = __fmaf_rn(6.0f, c, -ph);  // 6u = ph + pl exactly
+  d = __fsub_rn(s, ph);
+  const float ea = __fadd_rn(two_sum_err(xm, xp, tx), two_sum_err(ym, yp, ty));
+  const float eb = __fadd_rn(two_sum_err(zm, zp, tz), two_sum_err(tx, ty, ta));
+  const float ec = __fadd_rn(two_sum_err(ta, tz, s), __fsub_rn(two_sum_err(s, -ph, d), pl));
+  e = __fadd_rn(__fadd_rn(ea, eb), ec);
+  return fabsf(__fadd_rn(d, e)) <= 0x1.fffffep+127f;
+}
+// The same residual with every sum in FP64.
+__device__ __forceinline__ double resid_f64(float xm, float xp, float ym, float yp, float zm, float zp, float c) {
+  const double s = __dadd_rn(__dadd_rn(__dadd_rn(widen_f32(xm), widen_f32(xp)), __dadd_rn(widen_f32(ym), widen_f32(yp))),
+                             __dadd_rn(widen_f32(zm), widen_f32(zp)));
+  return __dsub_rn(s, __dmul_rn(6.0, widen_f32(c)));
+}
+
 // Spin (bounded by wall time `limit_ns` and by a poll count) until *flag >= target,
 // with acquire semantics.  Returns true on success.  On expiry it records
 // DEV_TIMEOUT in *err (first failure wins); it also gives up early when another

@@ -97,38 +97,47 @@ template <> struct V16<double> {
   }
 };
 
-// FP64 residual contribution of one point: r = s - 6u with s re-evaluated in
-// FP64 from the (exactly widened) neighbours in the stencil's order.  FP32
-// states are widened on the integer pipe, which leaves the slow FP64 pipe
-// only the additions and multiplications (same-box A/B: the 768^3 FP32
-// residual 10.5 -> 7.4 ms, the whole 200-iteration step with its residual
-// 684 -> 700 GLUP/s; residuals bit-identical).
-// r^2 for one point: r = s - 6u in FP64 (FP32 values widened exactly, the
-// neighbour sum recomputed in FP64 in the stencil's order).  With EMU (an
-// FP32 state inside the integer adder's domain: no sign bit, finite) the
-// three pair sums of the widened values run on the integer pipe (dadd_nn,
-// bit-identical to the FP64 pipe's addition there), which leaves the FP64
-// pipe five of its eight operations per point.  FP32 kernels use it only in
-// residual-only launches: same-box A/B, 768^3 residual 7.07 -> 5.87 ms,
-// while in the fused step-and-residual launches the extra code path spilled
-// (serving 84.0 -> 81.9 solves/s).
-template <typename T, bool EMU = false>
-__device__ __forceinline__ double resid2(T xm, T xp, T ym, T yp, T zm, T zp, T s, T c) {
-  double s64, c64;
-  if constexpr (sizeof(T) == 8) {
-    s64 = (double)s;
-    c64 = (double)c;
-  } else if constexpr (EMU) {
-    s64 = __dadd_rn(__dadd_rn(dadd_nn(widen_f32(xm), widen_f32(xp)), dadd_nn(widen_f32(ym), widen_f32(yp))),
-                    dadd_nn(widen_f32(zm), widen_f32(zp)));
-    c64 = widen_f32(c);
-  } else {
-    s64 = __dadd_rn(__dadd_rn(__dadd_rn(widen_f32(xm), widen_f32(xp)), __dadd_rn(widen_f32(ym), widen_f32(yp))),
-                    __dadd_rn(widen_f32(zm), widen_f32(zp)));
-    c64 = widen_f32(c);
+// Residual contributions r^2 of N neighbouring points, r = s - 6u in FP64 from
+// the state's values, added to acc in order; points with use[q] false add
+// nothing.  FP64: s is the stencil's own sum.  FP32: resid_split, FP64 sums only
+// where it cannot (one branch per vector): same-box, jacobi_residual at 768^3 in
+// 64^3 blocks 5.87 -> 2.08 ms, at 512^3 1.79 -> 0.67 ms, 32 served solves 550 ->
+// 540 ms, against sums of integer-widened values on the FP64 and integer pipes;
+// the norms are the same, and the step-and-residual kernels no longer spill.
+template <int N>
+__device__ __forceinline__ void resid_add(double& acc, const double (&)[N], const double (&)[N], const double (&)[N],
+                                          const double (&)[N], const double (&)[N], const double (&)[N], const double (&s)[N],
+                                          const double (&c)[N], const bool (&use)[N]) {
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const double r = __dsub_rn(s[q], __dmul_rn(6.0, c[q]));
+    acc += use[q] ? r * r : 0.0;
   }
-  const double r = __dsub_rn(s64, __dmul_rn(6.0, c64));
-  return r * r;
+}
+template <int N>
+__device__ __forceinline__ void resid_add(double& acc, const float (&xm)[N], const float (&xp)[N], const float (&ym)[N],
+                                          const float (&yp)[N], const float (&zm)[N], const float (&zp)[N], const float (&)[N],
+                                          const float (&c)[N], const bool (&use)[N]) {
+  double a = acc;
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    float d, e;
+    ok = resid_split(xm[q], xp[q], ym[q], yp[q], zm[q], zp[q], c[q], d, e) && ok;
+    double r = __dadd_rn(widen_f32(d), widen_f32(e));
+    if (!use[q]) r = 0.0;
+    a = fma(r, r, a);
+  }
+  if (!ok) {
+    a = acc;
+#pragma unroll 1
+    for (int q = 0; q < N; ++q) {
+      if (!use[q]) continue;
+      const double r = resid_f64(xm[q], xp[q], ym[q], yp[q], zm[q], zp[q], c[q]);
+      a = fma(r, r, a);
+    }
+  }
+  acc = a;
 }
 
 // ---------------------------------------------------------------------------
@@ -184,7 +193,11 @@ __device__ __forceinline__ double tile_sweep(const BlockDev& B, int p, int x0, i
         if (k == nz - 1 && szp) szp[col] = v;
       }
     }
-    if (MODE & kResid) acc += resid2<T>(xm, xp, ym, yp, below, above, s, cur);
+    if (MODE & kResid) {
+      const T a1[1] = {xm}, a2[1] = {xp}, a3[1] = {ym}, a4[1] = {yp}, a5[1] = {below}, a6[1] = {above}, a7[1] = {s}, a8[1] = {cur};
+      const bool use[1] = {true};
+      resid_add(acc, a1, a2, a3, a4, a5, a6, a7, a8, use);
+    }
     below = cur;
     cur = above;
   }
@@ -329,9 +342,7 @@ __device__ __forceinline__ double stream_plane(const PlaneView<T>& O, int k, int
                                                const unsigned char* sm, const unsigned char* sc,
                                                const unsigned char* sp, int tx, int j0) {
   constexpr int VEC = V16<T>::N;
-  // EMU: the integer-pipe adder takes the FP64 stencil's pair sums and, in
-  // either precision, the residual's (FP32 sums themselves stay FP32 adds)
-  constexpr bool EMU_SUM = EMU && sizeof(T) == 8;
+  constexpr bool EMU_SUM = EMU && sizeof(T) == 8;  // the integer-pipe adder takes the FP64 stencil's pair sums
   const int nx = O.nx, ny = O.ny, nz = O.nz;
   const int rx = RAG ? O.rx : nx, ry = RAG ? O.ry : ny;  // equal without padding
   const int i0 = tx * VEC;
@@ -402,11 +413,20 @@ __device__ __forceinline__ double stream_plane(const PlaneView<T>& O, int k, int
       // the loop made ptxas spill); FP32 finishes the vector after the loop
       // (one fallback branch per vector).
       if constexpr (sizeof(T) == 8) v[q] = finish1(s);
-      else sv[q] = s;
-      if (MODE & kResid) {
-        const double e2 = resid2<T, EMU>(xm, xp, ym[q], yp[q], zm[q], zp[q], s, c[r][q]);
-        acc += (!RAG || (q <= ql && j < ny)) ? e2 : 0.0;
+      if (sizeof(T) == 4 || (MODE & kResid)) sv[q] = s;
+    }
+    if (MODE & kResid) {
+      T xl[VEC], xr[VEC], yl[VEC], yr[VEC];
+      bool use[VEC];
+#pragma unroll
+      for (int q = 0; q < VEC; ++q) {
+        xl[q] = q == 0 ? left : c[r][q > 0 ? q - 1 : 0];
+        xr[q] = q == VEC - 1 ? right : c[r][q < VEC - 1 ? q + 1 : 0];
+        yl[q] = ym[q];
+        yr[q] = yp[q];
+        use[q] = !RAG || (q <= ql && j < ny);
       }
+      resid_add(acc, xl, xr, yl, yr, zm, zp, sv, c[r], use);
     }
     if constexpr (sizeof(T) == 4) finish_vec(sv, v);
     if ((MODE & kWrite) && (MODE & kPack)) {
@@ -479,7 +499,7 @@ __device__ double stream_item(const BlockDev& B, int p, const WorkItem& w, Ring&
   const StageLayout L = stage_layout<T>(B, w.ya, w.yb);
   PlaneView<T> O = plane_view<T>(B, p);
   O.ss = tab;
-  constexpr bool kEmuUse = sizeof(T) == 8 || MODE == kResid;  // FP32: residual-only launches
+  constexpr bool kEmuUse = sizeof(T) == 8;
   const int nplanes = w.z1 - w.z0 + 2;
   auto issue = [&](int q) {
     const int st = q % S;
@@ -660,7 +680,7 @@ __global__ void __launch_bounds__(StreamShape<CW>::threads, StreamShape<CW>::min
     }
   } else {
     // ---- consumers ----
-    const bool emu = (sizeof(T) == 8 || MODE == kResid) && a.emu && a.norms && a.norms[B.grid].emu_bad == 0u;
+    const bool emu = sizeof(T) == 8 && a.emu && a.norms && a.norms[B.grid].emu_bad == 0u;
     PlaneView<T> O = plane_view<T>(B, p);
     if (kSendTable) O.ss = s_send;
     const int txv = O.rx / VEC;
@@ -686,7 +706,7 @@ __global__ void __launch_bounds__(StreamShape<CW>::threads, StreamShape<CW>::min
         const unsigned char* sm = stages + (size_t)((q - 1) & Sm) * L.bytes;
         const unsigned char* sc = stages + (size_t)(q & Sm) * L.bytes;
         const unsigned char* sp = stages + (size_t)((q + 1) & Sm) * L.bytes;
-        if ((sizeof(T) == 8 || MODE == kResid) && emu)
+        if (sizeof(T) == 8 && emu)
           acc += stream_plane<T, RY, MODE, true, RAG, kSendTable, (CW < 8)>(O, w.z0 - 1 + q, w.ya, L, sm, sc, sp, tx, j0);
         else
           acc += stream_plane<T, RY, MODE, false, RAG, kSendTable, (CW < 8)>(O, w.z0 - 1 + q, w.ya, L, sm, sc, sp, tx, j0);
