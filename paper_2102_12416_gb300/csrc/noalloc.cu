@@ -23,30 +23,71 @@ namespace {
 
 constexpr int kMaxPlanes = JACOBI_NOALLOC_MAX_PLANES;
 constexpr int kNaThreads = 256;
+constexpr int kNaRows = 8;  // rows a warp walks with its y neighbours in registers
 
-// Two partials per z-plane: sum of r^2 and sum of b^2.
+// Two partials per CTA (a plane, or a share of its rows): sum of r^2, sum of b^2.
 static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxPlanes];
 
+// r = s - 6u of one point.  FP64: the pair sums on the integer pipe when all
+// lanes' neighbours are inside the adder's domain (the same rounded sums; the
+// two outer additions, 6u, the difference and the square stay on the FP64
+// pipe); FP32: resid_split.
+__device__ __forceinline__ double noalloc_r(double xm, double xp, double ym, double yp, double zm, double zp, double c, bool use) {
+  const uint32_t hi = max(max(max((uint32_t)__double2hiint(xm), (uint32_t)__double2hiint(xp)),
+                              max((uint32_t)__double2hiint(ym), (uint32_t)__double2hiint(yp))),
+                          max((uint32_t)__double2hiint(zm), (uint32_t)__double2hiint(zp)));
+  double sx, sy, sz;
+  if (__all_sync(0xffffffffu, !use || hi < kEmuHiLimit)) {
+    sx = dadd_nn(xm, xp);
+    sy = dadd_nn(ym, yp);
+    sz = dadd_nn(zm, zp);
+  } else {
+    sx = __dadd_rn(xm, xp);
+    sy = __dadd_rn(ym, yp);
+    sz = __dadd_rn(zm, zp);
+  }
+  return __dsub_rn(__dadd_rn(__dadd_rn(sx, sy), sz), __dmul_rn(6.0, c));
+}
+__device__ __forceinline__ double noalloc_r(float xm, float xp, float ym, float yp, float zm, float zp, float c, bool) {
+  float d, e;
+  if (resid_split(xm, xp, ym, yp, zm, zp, c, d, e)) return __dadd_rn(widen_f32(d), widen_f32(e));
+  return resid_f64(xm, xp, ym, yp, zm, zp, c);
+}
+
+// CTA (plane, share of its rows): its warps take strips of 32 columns x kNaRows
+// rows.  Bound by the FP64 pipe (FP64: 5 operations per point beside 3
+// integer-pipe sums, FP32: 2); the boundary sum is taken only at the points
+// that touch the boundary and the planes are split while they alone do not fill
+// the chip.  256^3 FP64: 528 us with both sums in FP64 at every point and one CTA
+// per plane, 262 us so.
 template <typename T>
-__global__ void __launch_bounds__(kNaThreads) k_noalloc_planes(const T* __restrict__ u, int64_t nx, int64_t ny,
-                                                             int64_t nz, double* scratch) {
-  const int64_t k = 1 + blockIdx.x;  // padded plane index
-  const int64_t px = nx + 2, py = ny + 2;
-  const int64_t n = nx * ny;
+__global__ void __launch_bounds__(kNaThreads) k_noalloc_planes(const T* __restrict__ u, int64_t nx, int64_t ny, int64_t nz,
+                                                             int split, double* scratch) {
+  const int64_t k = 1 + blockIdx.x / split;  // padded plane index
+  const int sub = blockIdx.x % split;
+  const int64_t px = nx + 2, pp = px * (ny + 2);
+  const int64_t j0 = 1 + ny * sub / split, j1 = 1 + ny * (sub + 1) / split;
+  const int lane = threadIdx.x & 31;
+  const int64_t cols = (nx + 31) / 32, tasks = cols * ((j1 - j0 + kNaRows - 1) / kNaRows);
   double ar = 0.0, ab = 0.0;
-  for (int64_t e = threadIdx.x; e < n; e += kNaThreads) {
-    const int64_t i = 1 + e % nx, j = 1 + e / nx;
-    const int64_t o = (k * py + j) * px + i;
-    const double w[6] = {(double)u[o - 1], (double)u[o + 1], (double)u[o - px],
-                         (double)u[o + px], (double)u[o - px * py], (double)u[o + px * py]};
-    const bool bnd[6] = {i == 1, i == nx, j == 1, j == ny, k == 1, k == nz};
-    double wb[6];
-    for (int q = 0; q < 6; ++q) wb[q] = bnd[q] ? w[q] : 0.0;
-    const double s = __dadd_rn(__dadd_rn(__dadd_rn(w[0], w[1]), __dadd_rn(w[2], w[3])), __dadd_rn(w[4], w[5]));
-    const double sb = __dadd_rn(__dadd_rn(__dadd_rn(wb[0], wb[1]), __dadd_rn(wb[2], wb[3])), __dadd_rn(wb[4], wb[5]));
-    const double r = __dsub_rn(s, __dmul_rn(6.0, (double)u[o]));
-    ar = fma(r, r, ar);
-    ab = fma(sb, sb, ab);
+  for (int64_t t = threadIdx.x >> 5; t < tasks; t += kNaThreads / 32) {
+    const int64_t i = 1 + (t % cols) * 32 + lane, ja = j0 + t / cols * kNaRows, jb = min(ja + kNaRows, j1);
+    const bool use = i <= nx;
+    const T* p = u + k * pp + ja * px + (use ? i : nx);  // lanes past the row reread its last point
+    T ym = p[-px], c = p[0];
+    for (int64_t j = ja; j < jb; ++j, p += px) {
+      const T yp = p[px], xm = p[-1], xp = p[1], zm = p[-pp], zp = p[pp];
+      const double r = noalloc_r(xm, xp, ym, yp, zm, zp, c, use);
+      if (use) ar = fma(r, r, ar);
+      if (use && (i == 1 || i == nx || j == 1 || j == ny || k == 1 || k == nz)) {
+        const double sb = __dadd_rn(__dadd_rn(__dadd_rn(i == 1 ? (double)xm : 0.0, i == nx ? (double)xp : 0.0),
+                                              __dadd_rn(j == 1 ? (double)ym : 0.0, j == ny ? (double)yp : 0.0)),
+                                    __dadd_rn(k == 1 ? (double)zm : 0.0, k == nz ? (double)zp : 0.0));
+        ab = fma(sb, sb, ab);
+      }
+      ym = c;
+      c = yp;
+    }
   }
   __shared__ double red[kNaThreads / 32];
   const double sr = block_sum<kNaThreads>(ar, red);
@@ -57,17 +98,16 @@ __global__ void __launch_bounds__(kNaThreads) k_noalloc_planes(const T* __restri
   }
 }
 
-// One warp: fixed-order sum of the plane partials, then |r|, |b|, rel.
-__global__ void k_noalloc_finish(const double* scratch, int64_t nz, double* out) {
+// One CTA: fixed-order sum of the partials, then |r|, |b|, rel.
+__global__ void __launch_bounds__(kNaThreads) k_noalloc_finish(const double* scratch, int n, double* out) {
   double r = 0.0, b = 0.0;
-  for (int64_t q = threadIdx.x; q < nz; q += 32) {
+  for (int q = threadIdx.x; q < n; q += kNaThreads) {
     r += scratch[2 * q];
     b += scratch[2 * q + 1];
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    r += __shfl_xor_sync(0xffffffffu, r, o);
-    b += __shfl_xor_sync(0xffffffffu, b, o);
-  }
+  __shared__ double red[kNaThreads / 32];
+  r = block_sum<kNaThreads>(r, red);
+  b = block_sum<kNaThreads>(b, red);
   if (threadIdx.x == 0) {
     const double rn = sqrt(r), bn = sqrt(b);
     out[0] = rn;
@@ -112,14 +152,17 @@ extern "C" int jacobi_residual_noalloc(const void* u_padded, jacobi_dim3 grid, j
   int rc = scratch_for_current_device(&scratch);
   if (rc) return rc;
   const cudaStream_t s = (cudaStream_t)stream;
+  // Shares per plane: about eight CTAs for each of 152 SMs, no less than kNaRows
+  // rows each, within the scratch array.
+  const int64_t split = std::max<int64_t>(1, std::min<int64_t>({(1216 + grid.nz - 1) / grid.nz, (grid.ny + kNaRows - 1) / kNaRows,
+                                                               kMaxPlanes / grid.nz}));
+  const unsigned ctas = (unsigned)(grid.nz * split);
   if (dtype == JACOBI_F64)
-    k_noalloc_planes<double><<<(unsigned)grid.nz, kNaThreads, 0, s>>>((const double*)u_padded, grid.nx, grid.ny, grid.nz,
-                                                                     scratch);
+    k_noalloc_planes<double><<<ctas, kNaThreads, 0, s>>>((const double*)u_padded, grid.nx, grid.ny, grid.nz, (int)split, scratch);
   else
-    k_noalloc_planes<float><<<(unsigned)grid.nz, kNaThreads, 0, s>>>((const float*)u_padded, grid.nx, grid.ny, grid.nz,
-                                                                    scratch);
+    k_noalloc_planes<float><<<ctas, kNaThreads, 0, s>>>((const float*)u_padded, grid.nx, grid.ny, grid.nz, (int)split, scratch);
   JGB_CUDA(cudaGetLastError());
-  k_noalloc_finish<<<1, 32, 0, s>>>(scratch, grid.nz, out);
+  k_noalloc_finish<<<1, kNaThreads, 0, s>>>(scratch, (int)ctas, out);
   JGB_CUDA(cudaGetLastError());
   return JACOBI_OK;
 }
