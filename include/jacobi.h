@@ -132,6 +132,14 @@ typedef struct { int32_t mode; int32_t pad_; int64_t x, y, z; } jacobi_split;
  *               through release/acquire progress flags in device memory
  *               instead of kernel boundaries (bounded waits).
  *   GRAPH:      the FUSED launches captured once in a CUDA graph and replayed.
+ * On GRAPH and PERSISTENT, a call of enough iterations (4 to some tens) on grids
+ * small enough to stay on chip (together about 1.3 M FP64 or 2.6 M FP32 points)
+ * runs as one cooperative launch of the resident kernel instead: boxes of the
+ * grids stay in shared memory and exchange their surfaces every iteration
+ * through packets in device memory (bounded waits, reported as on PERSISTENT);
+ * state and receive slots of the last iteration are written back.  The
+ * environment variable JACOBI_RESIDENT=0 at creation turns it off, as does a
+ * set JACOBI_PERSIST_WS; a stream under capture does not use it.
  * The next three run the halo exchange the way the paper's host-driven
  * runtimes do (Sec. 3, Sec. 4.3), for comparing the exchange forms on the
  * Jacobi3D workload; each iteration is a stencil launch followed by the

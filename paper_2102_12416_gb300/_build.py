@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libjacobi_gb300.so")
-SOURCES = ["kernels.cu", "step.cu", "api.cu", "channel.cu", "serve.cu", "noalloc.cu"]
+SOURCES = ["kernels.cu", "step.cu", "api.cu", "channel.cu", "serve.cu", "noalloc.cu", "resident.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
               "-Xcompiler", "-fPIC,-O2", "-Xptxas", "-v", "--expt-relaxed-constexpr"]
 

@@ -229,6 +229,29 @@ int plan_items(Plan* P, int64_t zc_req, int cw_cap, int64_t target_items, int64_
   return JACOBI_OK;
 }
 
+ResGrid resident_grid(const GridHost& G, int32_t index) {
+  ResGrid r{};
+  r.grid = index;
+  r.block0 = (int32_t)G.block_begin;
+  r.mode = G.split.mode == JACOBI_SPLIT_SHAPE ? 1 : 0;
+  const int64_t n[3] = {G.dims.nx, G.dims.ny, G.dims.nz}, q[3] = {G.split.x, G.split.y, G.split.z};
+  for (int d = 0; d < 3; ++d) {
+    r.n[d] = (int32_t)n[d];
+    r.param[d] = (int32_t)std::min<int64_t>(q[d], 1 << 30);
+    r.cnt[d] = (int32_t)G.counts[d];
+  }
+  return r;
+}
+
+ResLayout resident_layout(const ResPlan& rp, size_t n_grids) {
+  ResLayout L;
+  L.grids = align_up(rp.boxes.size() * sizeof(ResBox), 256);
+  L.ctl = align_up(L.grids + n_grids * sizeof(ResGrid), 256);
+  L.packets = L.ctl + 256;
+  L.bytes = L.packets + rp.packet_units * 16;
+  return L;
+}
+
 int plan_build(int64_t n_grids, const jacobi_dim3* grids, const jacobi_split* splits, jacobi_dtype dtype,
                const jacobi_init* inits, Plan* P, int64_t target_items, int64_t min_chunk) {
   if (n_grids < 1 || !grids || !splits) return set_error(JACOBI_EINVAL, "need at least one grid");
@@ -346,6 +369,13 @@ int plan_build(int64_t n_grids, const jacobi_dim3* grids, const jacobi_split* sp
   P->off_active_blocks = take(nb * sizeof(int32_t));
   P->off_it0 = take(sizeof(int64_t));
   P->off_ticket = take(sizeof(unsigned long long));
+  // Resident path of a handle (the server's requests share step launches).
+  if (target_items <= 0 && n_grids <= device_sms()) {
+    std::vector<ResGrid> rg;
+    for (int64_t g = 0; g < n_grids; ++g) rg.push_back(resident_grid(P->grids[g], (int32_t)g));
+    ResPlan rp;
+    if (resident_plan(rg, dtype, (int)device_sms(), &rp)) P->res_bytes = resident_layout(rp, rg.size()).bytes;
+  }
   const size_t per16 = 32;  // plane pitch rounded to 32 elements
   for (auto& B : P->blocks) {
     B.pitch = (int64_t)align_up((size_t)(B.rx * B.ry), per16);
@@ -454,6 +484,47 @@ int upload_tables(jacobi_t* h, cudaStream_t s) {
   return JACOBI_OK;
 }
 
+// Boxes and packet buffers of the resident path for the active grids; without
+// them (they do not fit, or there is no memory) the other kernels run.
+int build_resident(jacobi_t* h, cudaStream_t s) {
+  Resident& R = h->res;
+  R.ok = false;
+  if (!R.allowed || h->plan.res_bytes == 0) return JACOBI_OK;
+  const Plan& P = h->plan;
+  std::vector<ResGrid> grids;
+  for (int32_t g : h->active_grids) grids.push_back(resident_grid(P.grids[g], g));
+  ResPlan rp;
+  if (!resident_plan(grids, P.dtype, (int)device_sms(), &rp) || rp.iter_ns >= rp.launch_ns) return JACOBI_OK;
+  R.min_iters = std::max<int64_t>(4, (int64_t)std::ceil(rp.once_ns / (rp.launch_ns - rp.iter_ns)));
+  const ResLayout L = resident_layout(rp, grids.size());
+  char* mem = R.with_ws;
+  if (!mem || L.bytes > P.res_bytes) {
+    if (L.bytes > R.own_bytes) {
+      if (R.own) cudaFree(R.own);  // (synchronises; the tables are being replaced anyway)
+      R.own = nullptr;
+      R.own_bytes = 0;
+      if (cudaMalloc((void**)&R.own, L.bytes) != cudaSuccess) {
+        cudaGetLastError();
+        R.own = nullptr;
+        return JACOBI_OK;
+      }
+      R.own_bytes = L.bytes;
+    }
+    mem = R.own;
+  }
+  R.d_boxes = (ResBox*)mem;
+  R.d_grids = (ResGrid*)(mem + L.grids);
+  R.d_ctl = (uint32_t*)(mem + L.ctl);
+  R.d_packets = (uint4*)(mem + L.packets);
+  JGB_CUDA(cudaMemcpyAsync(R.d_boxes, rp.boxes.data(), rp.boxes.size() * sizeof(ResBox), cudaMemcpyHostToDevice, s));
+  JGB_CUDA(cudaMemcpyAsync(R.d_grids, grids.data(), grids.size() * sizeof(ResGrid), cudaMemcpyHostToDevice, s));
+  JGB_CUDA(cudaMemsetAsync(R.d_ctl, 0, L.bytes - L.ctl, s));  // no packet of the old tables may match a number
+  R.n_boxes = (int)rp.boxes.size();
+  R.smem = rp.smem;
+  R.ok = true;
+  return JACOBI_OK;
+}
+
 // Rebuild the active item / block lists from the grids' active flags.
 int refresh_active(jacobi_t* h, cudaStream_t s) {
   if (!h->tables_dirty) return JACOBI_OK;
@@ -539,6 +610,8 @@ int refresh_active(jacobi_t* h, cudaStream_t s) {
     h->h_grids[g].active = 1;  // inactive grids have no items in the launch lists
   }
   JGB_CUDA(cudaMemcpyAsync(h->d_grids, h->h_grids, P.grids.size() * sizeof(GridDev), cudaMemcpyHostToDevice, s));
+  const int rcr = build_resident(h, s);
+  if (rcr) return rcr;
   JGB_CUDA(cudaStreamSynchronize(s));  // host mirrors are reused below
   h->tables_dirty = false;
   return JACOBI_OK;
@@ -855,12 +928,53 @@ int step_exchange(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s, cudaEvent
   return JACOBI_OK;
 }
 
+// The resident kernel takes calls of res.min_iters iterations or more on the
+// GRAPH and PERSISTENT paths when the active grids fit.  Not under stream
+// capture (the cooperative launch would have to be marked in the caller's
+// graph), nor with an injected fault or redirected faces, which are about the
+// other kernels' exchange.
+bool resident_applies(const jacobi_t* h, int64_t n, cudaStream_t s) {
+  if (!h->res.ok || n < h->res.min_iters || h->drop_block >= 0 || h->local_halo ||
+      (h->path != JACOBI_PATH_GRAPH && h->path != JACOBI_PATH_PERSISTENT))
+    return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+}
+
+int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
+  const Resident& R = h->res;
+  ResLaunch a{};
+  a.blocks = h->d_blocks;
+  a.boxes = R.d_boxes;
+  a.rgrids = R.d_grids;
+  a.grids = h->d_grids;
+  a.norms = h->d_norms;
+  a.packets = R.d_packets;
+  a.ctl = R.d_ctl;
+  a.err = h->d_err;
+  a.wait_ns = h->wait_ns;
+  a.it0 = it0;
+  a.n_iters = n;
+  a.n_boxes = R.n_boxes;
+  a.smem = R.smem;
+  a.dtype = h->plan.dtype;
+  a.emu = h->fp64_emu;
+  JGB_CUDA(launch_resident(a, s));
+  return JACOBI_OK;
+}
+
 // Advance active grids by n iterations on the selected path.
 int do_step(jacobi_t* h, int64_t n, cudaStream_t s) {
   int rc = refresh_active(h, s);
   if (rc) return rc;
   if (n <= 0 || h->active_items.empty()) {
     h->iter += std::max<int64_t>(n, 0);
+    return JACOBI_OK;
+  }
+  if (resident_applies(h, n, s)) {
+    rc = step_resident(h, h->iter, n, s);
+    if (rc) return rc;
+    h->iter += n;
     return JACOBI_OK;
   }
   switch (h->path) {
@@ -1088,6 +1202,7 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
   const cudaStream_t s = S(stream);
   auto fail = [&](int code) {
     kind_fork_destroy(&h->fork);
+    if (h->res.own) cudaFree(h->res.own);
     if (h->own_ws && h->ws) cudaFree(h->ws);
     if (h->h_grids) cudaFreeHost(h->h_grids);
     if (h->h_norms) cudaFreeHost(h->h_norms);
@@ -1105,12 +1220,15 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
     if ((uintptr_t)workspace % 256) return fail(set_error(JACOBI_EINVAL, "workspace must be 256-byte aligned"));
     h->ws = (char*)workspace;
   } else {
-    e = cudaMalloc((void**)&h->ws, h->plan.bytes);
+    // (the resident path's tables, at most a few MB, follow the workspace)
+    const size_t ws_end = align_up(h->plan.bytes, 256);
+    e = cudaMalloc((void**)&h->ws, ws_end + h->plan.res_bytes);
     if (e != cudaSuccess) {
       h->ws = nullptr;
       return fail(set_error(JACOBI_ENOMEM, "cudaMalloc(%zu) failed: %s", h->plan.bytes, cudaGetErrorString(e)));
     }
     h->own_ws = true;
+    h->res.with_ws = h->ws + ws_end;
   }
   if (cudaMallocHost((void**)&h->h_grids, h->plan.grids.size() * sizeof(GridDev)) != cudaSuccess ||
       cudaMallocHost((void**)&h->h_norms, h->plan.grids.size() * sizeof(GridNorm)) != cudaSuccess ||
@@ -1146,7 +1264,11 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
   // pick another); the per-step kernels always use kStreamStages.
   h->stages = 4;
   if (const char* em = getenv("JACOBI_FP64_EMU")) h->fp64_emu = atoi(em) != 0 ? 1 : 0;
-  if (const char* pw = getenv("JACOBI_PERSIST_WS")) h->persist_ws = atoi(pw) != 0;
+  if (const char* pw = getenv("JACOBI_PERSIST_WS")) {
+    h->persist_ws = atoi(pw) != 0;
+    h->res.allowed = false;  // a persistent kernel was asked for by name
+  }
+  if (const char* rs = getenv("JACOBI_RESIDENT")) h->res.allowed = atoi(rs) != 0;
   if (const char* st = getenv("JACOBI_STAGES")) {
     const int v = atoi(st);
     if (v >= 3 && v <= 8) {
@@ -1186,6 +1308,7 @@ int jacobi_destroy(jacobi_t* h) {
   for (auto& pg : h->pgraph)
     if (pg.exec) cudaGraphExecDestroy(pg.exec);
   kind_fork_destroy(&h->fork);
+  if (h->res.own) cudaFree(h->res.own);
   if (h->stage) cudaFree(h->stage);
   if (h->d_desc) cudaFree(h->d_desc);
   if (h->h_desc) cudaFreeHost(h->h_desc);
@@ -1489,7 +1612,7 @@ int jacobi_step_timed(jacobi_t* h, int64_t n_iters, void* stream, double* comput
     float a = 0.f;
     if (!rc) cudaEventElapsedTime(&a, ev[0], ev[1]);
     comp = a;
-    if (!rc && h->path == JACOBI_PATH_PERSISTENT) rc = check_err_word(h, s);
+    if (!rc && (h->path == JACOBI_PATH_PERSISTENT || h->res.ok)) rc = check_err_word(h, s);
   }
   destroy();
   if (rc) return rc;
@@ -1537,7 +1660,7 @@ int jacobi_solve(jacobi_t* h, double tol, int64_t max_iters, int64_t check_every
       if (rc) return rc;
       rc = read_norms(h, s);
       if (rc) return rc;
-      if (h->path == JACOBI_PATH_PERSISTENT) {
+      if (h->path == JACOBI_PATH_PERSISTENT || h->res.ok) {
         rc = check_err_word(h, s);
         if (rc) return rc;
       }

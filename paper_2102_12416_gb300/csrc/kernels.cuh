@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "common.cuh"
 
@@ -179,5 +180,55 @@ inline int persistent_threads(const WorkItem* items, size_t n) {
   for (size_t i = 0; i < n; ++i) t = std::max(t, items[i].x0 >= 0 ? 256 : 32 * (items[i].y0 & 15));
   return t;
 }
+
+// Resident path (resident.cu): one cooperative launch runs n_iters iterations
+// with every box of the active grids in the shared memory of a CTA of its own.
+constexpr int kResSmem = 227 * 1024 - 1024;  // beside a little static shared memory
+
+// One grid: where its blocks stand in the device table, and how its axes are split.
+struct ResGrid {
+  int32_t grid;      // index in the device grid table
+  int32_t block0;    // its first block
+  int32_t mode;      // split mode (0: count, 1: extent)
+  int32_t n[3];      // interior points
+  int32_t param[3];  // blocks per axis, or block extent
+  int32_t cnt[3];    // blocks per axis
+};
+// One box: grid points [o, o + n) of a grid, its incoming packet buffer and where
+// its faces go (16-byte units from the packet buffer's start; the buffer of odd
+// iterations follows that of even ones).
+struct ResBox {
+  int32_t rgrid;
+  int32_t o[3], n[3];
+  int32_t faces;                      // bit f: the box across face f belongs to the grid
+  int32_t n_vec, n_one;               // incoming entries: 16-byte vectors (two units), x values (one)
+  uint32_t in_base, in_units;
+  uint32_t out_base[6], out_units[6];
+};
+struct ResPlan {
+  std::vector<ResBox> boxes;
+  size_t packet_units = 0;
+  int smem = 0;
+  // estimates: the launch without its iterations, an iteration, and an iteration
+  // as a launch of its own
+  double once_ns = 0.0, iter_ns = 0.0, launch_ns = 0.0;
+};
+// Cut grids into at most n_ctas boxes; false when they do not fit.
+bool resident_plan(const std::vector<ResGrid>& grids, int dtype, int n_ctas, ResPlan* P);
+
+struct ResLaunch {
+  const BlockDev* blocks;
+  const ResBox* boxes;
+  const ResGrid* rgrids;
+  const GridDev* grids;
+  const GridNorm* norms;  // per-grid emu_bad flags
+  uint4* packets;
+  uint32_t* ctl;          // [0] next sequence number, [1] CTAs that have finished
+  uint32_t* err;
+  uint64_t wait_ns;
+  int64_t it0, n_iters;
+  int32_t n_boxes, smem, dtype, emu;
+};
+cudaError_t launch_resident(const ResLaunch& a, cudaStream_t s);
 
 }  // namespace jgb

@@ -71,6 +71,7 @@ struct Plan {
   size_t off_blocks, off_geom, off_items, off_active, off_kind, off_grids, off_norms, off_inits, off_gids, off_partials,
       off_progress, off_err, off_stage_tab, off_punit_items, off_punit_ids, off_pdep_off, off_pdep_ids,
       off_active_blocks, off_it0, off_ticket;
+  size_t res_bytes = 0;    // resident-path tables and packets of a handle whose grids fit (not part of `bytes`)
   size_t off_stage_begin = 0, off_stage_end = 0;  // the explicit-path staging buffers, contiguous
   int64_t halo_faces = 0;                         // internal faces (one message each per iteration)
   size_t bytes = 0;
@@ -92,6 +93,14 @@ int plan_build(int64_t n_grids, const jacobi_dim3* grids, const jacobi_split* sp
 // 0 = the cost model's; at most cw_cap consumer warps per streaming CTA).
 int plan_items(Plan* P, int64_t zc_req, int cw_cap, int64_t target_items, int64_t min_chunk);
 
+// Resident path: a plan's grid as resident_plan takes it, and the layout of its
+// tables and packets (byte offsets).
+struct ResLayout {
+  size_t grids, ctl, packets, bytes;
+};
+ResGrid resident_grid(const GridHost& G, int32_t index);
+ResLayout resident_layout(const ResPlan& rp, size_t n_grids);
+
 // Device block table entries of a plan whose workspace starts at `ws`; block
 // and neighbour ids are offset by `base`; grid_override >= 0 replaces every
 // block's grid index.  stage_tab (nullable) receives the explicit-path staging
@@ -99,6 +108,28 @@ int plan_items(Plan* P, int64_t zc_req, int cw_cap, int64_t target_items, int64_
 // receive slots instead of its neighbours' (the halo-share measurement).
 void fill_block_tables(const Plan& P, char* ws, int64_t base, int32_t grid_override, BlockDev* bd, BlockGeom* geo,
                        void** stage_tab, bool local_halo = false);
+
+}  // namespace jgb
+
+namespace jgb {
+
+// Resident-path tables of one handle (resident.cu), rebuilt with the active
+// lists: behind a workspace of the library's own, or in memory of their own
+// beside a caller's or when a subset of the grids needs more than all did (its
+// boxes are smaller and more).
+struct Resident {
+  bool allowed = true;   // off when the environment asks for a given persistent kernel
+  bool ok = false;       // the active grids fit
+  int n_boxes = 0, smem = 0;
+  int64_t min_iters = 0; // shortest call it takes
+  char* with_ws = nullptr;
+  char* own = nullptr;
+  size_t own_bytes = 0;
+  ResBox* d_boxes = nullptr;
+  ResGrid* d_grids = nullptr;
+  uint32_t* d_ctl = nullptr;
+  uint4* d_packets = nullptr;
+};
 
 }  // namespace jgb
 
@@ -151,6 +182,7 @@ struct jacobi_s {
   jgb::GridNorm* h_norms = nullptr;  // pinned, read back from d_norms
   uint32_t* h_err = nullptr;        // pinned
 
+  jgb::Resident res;              // small problems: all iterations of a call on chip
   jgb::KindFork fork;             // side-by-side launch of the step's item kinds
   // CUDA graph of the fused path
   cudaGraphExec_t graph = nullptr;

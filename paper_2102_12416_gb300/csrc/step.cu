@@ -22,6 +22,7 @@
 //  * tiles (x0 >= 0): a TX x TY tile of columns, one column per thread, read
 //    straight from global memory with the z neighbours in registers.
 #include "kernels.cuh"
+#include "stencil.cuh"
 
 namespace jgb {
 
@@ -73,29 +74,6 @@ __device__ __noinline__ bool mbar_wait(uint64_t* b, uint32_t parity, uint32_t* e
 __device__ __forceinline__ bool mbar_ready(uint64_t* b, uint32_t parity, uint32_t* err, uint64_t limit_ns) {
   return mbar_test(b, parity) || mbar_wait(b, parity, err, limit_ns);
 }
-
-// ---- 16-byte vectors ---------------------------------------------------------
-template <typename T> struct V16;
-template <> struct V16<float> {
-  static constexpr int N = 4;
-  __device__ static __forceinline__ void load(const float* p, float (&v)[4]) {
-    const float4 x = *reinterpret_cast<const float4*>(p);
-    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-  }
-  __device__ static __forceinline__ void store(float* p, const float (&v)[4]) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-  }
-};
-template <> struct V16<double> {
-  static constexpr int N = 2;
-  __device__ static __forceinline__ void load(const double* p, double (&v)[2]) {
-    const double2 x = *reinterpret_cast<const double2*>(p);
-    v[0] = x.x; v[1] = x.y;
-  }
-  __device__ static __forceinline__ void store(double* p, const double (&v)[2]) {
-    *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
-  }
-};
 
 // Residual contributions r^2 of N neighbouring points, r = s - 6u in FP64 from
 // the state's values, added to acc in order; points with use[q] false add
@@ -213,32 +191,6 @@ struct Ring {
   int S;
   uint32_t pbits;  // parity of each stage's next fill (bit st), barrier-driven form only
 };
-
-// Sum of the six neighbours in the stencil's order.  With EMU (FP64 states
-// inside the integer adder's domain) the three pair sums run on the integer
-// pipe and the two outer additions on the FP64 pipe: both pipes share the
-// work and the result is bit-identical.
-template <typename T, bool EMU>
-__device__ __forceinline__ T nsum(T xm, T xp, T ym, T yp, T zm, T zp) {
-  if (EMU) {
-    const double sx = dadd_nn((double)xm, (double)xp), sy = dadd_nn((double)ym, (double)yp),
-                 sz = dadd_nn((double)zm, (double)zp);
-    return (T)__dadd_rn(__dadd_rn(sx, sy), sz);
-  }
-  return radd(radd(radd(xm, xp), radd(ym, yp)), radd(zm, zp));
-}
-
-// nsum with the z pair on the FP64 pipe (bit-identical: both adders round
-// to nearest-even).
-template <typename T, bool EMU>
-__device__ __forceinline__ T nsum_zn(T xm, T xp, T ym, T yp, T zm, T zp) {
-  if (EMU) {
-    const double sx = dadd_nn((double)xm, (double)xp), sy = dadd_nn((double)ym, (double)yp),
-                 sz = __dadd_rn((double)zm, (double)zp);
-    return (T)__dadd_rn(__dadd_rn(sx, sy), sz);
-  }
-  return radd(radd(radd(xm, xp), radd(ym, yp)), radd(zm, zp));
-}
 
 // Shared-memory stage of one plane of a padded row window [ya, yb) of block
 // B: rows ra..rb-1 of the plane (the window plus one neighbour row on each
