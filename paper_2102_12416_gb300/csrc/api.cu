@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 
 #include "runtime.h"
 
@@ -97,31 +98,53 @@ static int64_t device_sms() {
   return 152;
 }
 
-// z-chunk of a handle's work items by a cost model: a launch takes
-// ceil(items / C) waves of C resident CTAs, each item costs its planes plus a
-// fixed pipeline fill of ~2 planes, and in FP32 (bound by memory, not by
-// arithmetic) each chunk's two re-read halo planes cost about one plane of
-// traffic.  C counts the CTAs of the kind with the most units.  Candidates
-// halve from the tallest block down to zmin planes; ties keep the longer chunk.
-// FP32 chunks start at 32 planes at most: on 768^3 in 64^3 blocks, 64-plane
-// chunks measured ~2 % slower than 32 although the model prefers them.
+// z-chunk of a handle's work items by a cost model over the CTAs of the kind
+// with the most units.
+//
+// FP64 (bound by arithmetic): an SM gets ceil(items / SMs) CTAs and runs r of
+// them (its resident limit) at a time; a plane of k running CTAs takes k times
+// its points at 1.0 ns, but no less than the 2.5 us of one CTA alone; a chunk
+// costs 0.15 planes more, a launch 5.7 us.  Fitted to 200 timings of 14 problems
+// of 96^3 .. 512^3 points over z-chunks of 1 .. 64 (rms 5 %), whose best chunk
+// it finds to 1 % (192^3 in 32^3 blocks: 7 %); counting waves of equal CTAs instead,
+// as for FP32, was up to 20 % slower between them: 224^3 in 64^3 blocks 105 ->
+// 123 GLUP/s, 9 grids of 96^3 103 -> 123, 301x203x157 in 60^3 blocks 85 -> 97.
+//
+// FP32 (bound by memory) and tiles: a launch takes ceil(items / C) waves of C
+// resident CTAs, each item costs its planes plus a fixed pipeline fill of ~2
+// planes, and in FP32 each chunk's two re-read halo planes cost about one plane
+// of traffic.  FP32 chunks start at 32 planes at most: on 768^3 in 64^3 blocks,
+// 64-plane chunks measured ~2 % slower than 32 although the model prefers them.
+//
+// FP32 candidates halve from the tallest block down to zmin planes, FP64 ones are
+// these and every depth up to 16; ties keep the longer chunk.
 static int64_t choose_chunk(const Plan& P, const std::vector<int>& warps, const std::vector<int64_t>& chunks,
                             int64_t maxz, int64_t zmin) {
   int64_t kind_units[4] = {0, 0, 0, 0};  // tiles, CW 8, 4, 2
+  int64_t kind_area[4] = {0, 0, 0, 0};   // points of a plane of its largest window
   for (size_t b = 0; b < P.blocks.size(); ++b) {
     const BlockHost& B = P.blocks[b];
     const int cw = warps[b];
     const int k = cw == 0 ? 0 : cw == 8 ? 1 : cw == 4 ? 2 : 3;
     kind_units[k] += cw ? (B.ry + chunks[b] - 1) / chunks[b] : ((B.extent[0] + TX - 1) / TX) * ((B.extent[1] + TY - 1) / TY);
+    kind_area[k] = std::max(kind_area[k], B.rx * chunks[b]);
   }
   const int k = (int)(std::max_element(kind_units, kind_units + 4) - kind_units);
   const int64_t per_sm = k == 0 ? 8 : stream_ctas_per_sm(k == 1 ? 8 : k == 2 ? 4 : 2, P.max_stage);
-  const int64_t C = device_sms() * per_sm;
+  const int64_t sms = device_sms(), C = sms * per_sm;
+  const bool f64 = P.dtype == JACOBI_F64 && k > 0;
   const double halo = P.dtype == JACOBI_F32 ? 1.0 : 0.0;
   const int64_t z0 = P.dtype == JACOBI_F32 ? std::max<int64_t>(std::min<int64_t>(maxz, 32), zmin) : maxz;
-  int64_t best = z0;
-  double best_cost = 0.0;
+  std::vector<int64_t> cand;
   for (int64_t zc = z0;; zc = (zc + 1) / 2) {
+    cand.push_back(zc);
+    if (zc <= zmin || (zc + 1) / 2 < zmin) break;
+  }
+  for (int64_t zc = std::min<int64_t>(maxz, 16); f64 && zc >= zmin; --zc) cand.push_back(zc);
+  std::sort(cand.begin(), cand.end(), std::greater<int64_t>());
+  int64_t best = z0;
+  double best_cost = INFINITY;
+  for (int64_t zc : cand) {
     int64_t items = 0;
     for (size_t b = 0; b < P.blocks.size(); ++b) {
       const BlockHost& B = P.blocks[b];
@@ -129,13 +152,20 @@ static int64_t choose_chunk(const Plan& P, const std::vector<int>& warps, const 
                                          : ((B.extent[0] + TX - 1) / TX) * ((B.extent[1] + TY - 1) / TY);
       items += per_plane * ((B.extent[2] + zc - 1) / zc);
     }
-    const double waves = (double)((items + C - 1) / C);
-    const double cost = waves * ((double)zc + 2.0) * (1.0 + halo / (double)zc);
-    if (zc == z0 || cost < best_cost) {
+    double cost;
+    if (f64) {
+      const int64_t m = (items + sms - 1) / sms;
+      const double plane = 1e-3 * (double)kind_area[k];  // us of one CTA's plane at the SM's rate
+      cost = 5.7 + ((double)zc + 0.15) * ((double)(m / per_sm) * std::max(2.5, (double)per_sm * plane) +
+                                          (m % per_sm ? std::max(2.5, (double)(m % per_sm) * plane) : 0.0));
+    } else {
+      const double waves = (double)((items + C - 1) / C);
+      cost = waves * ((double)zc + 2.0) * (1.0 + halo / (double)zc);
+    }
+    if (cost < best_cost) {
       best = zc;
       best_cost = cost;
     }
-    if (zc <= zmin || (zc + 1) / 2 < zmin) break;
   }
   return best;
 }
