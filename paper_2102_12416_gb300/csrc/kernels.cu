@@ -397,12 +397,16 @@ __global__ void __launch_bounds__(kThreads) k_bnorm(StepLaunch a) {
   if (threadIdx.x == 0) a.partials[w.slot] = s;
 }
 
-// Self-test of the integer-pipe adder: out[i] = dadd_nn(a[i], b[i]).
+// Self-test of the integer-pipe adders: out[i] = a[i] + b[i] by dadd_nn, or NaN
+// where dadd_near reaches (a sum with zero included) and differs from it.
 __global__ void k_selftest_dadd(const double* a, const double* b, int64_t n, double* out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t j = i < n ? i : n - 1;  // clamped index: every lane loads in bounds
-  const double r = dadd_nn(a[j], b[j]);
-  if (i < n) out[i] = r;
+  int far = 0;
+  const double r = dadd_nn(a[j], b[j]), r2 = dadd_near(a[j], b[j], far);
+  if (far < 0) far = exp_far(a[j], b[j], 10);
+  const bool same = far < 0 || __double_as_longlong(r) == __double_as_longlong(r2);
+  if (i < n) out[i] = same ? r : __longlong_as_double(-1ll);
 }
 
 // Every binary32 bit pattern through widen_f32, against the conversion

@@ -28,25 +28,28 @@ constexpr int kNaRows = 8;  // rows a warp walks with its y neighbours in regist
 // Two partials per CTA (a plane, or a share of its rows): sum of r^2, sum of b^2.
 static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxPlanes];
 
-// r = s - 6u of one point.  FP64: the pair sums on the integer pipe when all
-// lanes' neighbours are inside the adder's domain (the same rounded sums; the
-// two outer additions, 6u, the difference and the square stay on the FP64
-// pipe); FP32: resid_split.
+// r = s - 6u of one point.  FP64: four of the five sums on the integer pipe when
+// all lanes' neighbours are inside the adders' domain (the same rounded sums, by
+// dadd_near, or dadd_nn where some lane's are out of its reach; the last sum, 6u,
+// the difference and the square stay on the FP64 pipe).  FP32: resid_split.
 __device__ __forceinline__ double noalloc_r(double xm, double xp, double ym, double yp, double zm, double zp, double c, bool use) {
   const uint32_t hi = max(max(max((uint32_t)__double2hiint(xm), (uint32_t)__double2hiint(xp)),
                               max((uint32_t)__double2hiint(ym), (uint32_t)__double2hiint(yp))),
                           max((uint32_t)__double2hiint(zm), (uint32_t)__double2hiint(zp)));
-  double sx, sy, sz;
+  double sxy, sz;
   if (__all_sync(0xffffffffu, !use || hi < kEmuHiLimit)) {
-    sx = dadd_nn(xm, xp);
-    sy = dadd_nn(ym, yp);
-    sz = dadd_nn(zm, zp);
+    int far = 0;
+    sxy = dadd_near(dadd_near(xm, xp, far), dadd_near(ym, yp, far), far);
+    sz = dadd_near(zm, zp, far);
+    if (__any_sync(0xffffffffu, use && far < 0 && sum_far(xm, xp, ym, yp, zm, zp, true) < 0)) {
+      sxy = dadd_nn(dadd_nn(xm, xp), dadd_nn(ym, yp));
+      sz = dadd_nn(zm, zp);
+    }
   } else {
-    sx = __dadd_rn(xm, xp);
-    sy = __dadd_rn(ym, yp);
+    sxy = __dadd_rn(__dadd_rn(xm, xp), __dadd_rn(ym, yp));
     sz = __dadd_rn(zm, zp);
   }
-  return __dsub_rn(__dadd_rn(__dadd_rn(sx, sy), sz), __dmul_rn(6.0, c));
+  return __dsub_rn(__dadd_rn(sxy, sz), __dmul_rn(6.0, c));
 }
 __device__ __forceinline__ double noalloc_r(float xm, float xp, float ym, float yp, float zm, float zp, float c, bool) {
   float d, e;
@@ -55,11 +58,11 @@ __device__ __forceinline__ double noalloc_r(float xm, float xp, float ym, float 
 }
 
 // CTA (plane, share of its rows): its warps take strips of 32 columns x kNaRows
-// rows.  Bound by the FP64 pipe (FP64: 5 operations per point beside 3
+// rows.  Bound by the FP64 pipe (FP64: 4 operations per point beside 4
 // integer-pipe sums, FP32: 2); the boundary sum is taken only at the points
 // that touch the boundary and the planes are split while they alone do not fill
 // the chip.  256^3 FP64: 528 us with both sums in FP64 at every point and one CTA
-// per plane, 262 us so.
+// per plane, 238 us so.
 template <typename T>
 __global__ void __launch_bounds__(kNaThreads) k_noalloc_planes(const T* __restrict__ u, int64_t nx, int64_t ny, int64_t nz,
                                                              int split, double* scratch) {

@@ -12,8 +12,8 @@
 // that finds the number has the payload, and no fence, flag or release is needed.
 // What an iteration costs beside its arithmetic is one store -> L2 -> load trip
 // and one CTA barrier.  Per iteration, launch path -> resident: 32^3 5.1 -> 1.7 us
-// (FP32) and 5.7 -> 2.0 (FP64), 64^3 FP64 6.7 -> 4.5, 96^3 FP32 5.6 -> 3.0 and FP64
-// 11.2 -> 8.6, 128^3 FP32 6.4 -> 5.2; a call costs about 14 us once (launch,
+// (FP32) and 5.7 -> 2.0 (FP64), 64^3 FP64 6.7 -> 4.2, 96^3 FP32 5.6 -> 3.0 and FP64
+// 11.2 -> 7.9, 128^3 FP32 6.4 -> 5.2; a call costs about 14 us once (launch,
 // tables, the state's way in and out).
 //
 // Boxes: each active grid is cut into cx * cy * cz near-equal boxes (x cuts on
@@ -101,16 +101,37 @@ template <> struct Words<double> {
 };
 
 // One update of a vector from its neighbours (the step kernels' arithmetic).
+// FP64 inside the integer adders' domain: pair sums by dadd_near, and xy of one of
+// the two points too (the pipes retire 836 and 527 G additions/s); a vector with
+// operands out of its reach is computed again with dadd_nn.  64^3 4.5 -> 4.2 us per
+// iteration, 108^3 11.4 -> 10.0, against dadd_nn alone.  `whole`: the second value
+// belongs to the grid.
 template <bool EMU>
 __device__ __forceinline__ void update(const double (&c)[2], const double (&ym)[2], const double (&yp)[2], const double (&zm)[2],
-                                       const double (&zp)[2], double left, double right, double (&v)[2]) {
-  // as in the streaming kernels, some z pairs go to the FP64 pipe
-  v[0] = finish1(nsum<double, EMU>(left, c[1], ym[0], yp[0], zm[0], zp[0]));
-  v[1] = finish1(nsum_zn<double, EMU>(c[0], right, ym[1], yp[1], zm[1], zp[1]));
+                                       const double (&zp)[2], double left, double right, bool whole, double (&v)[2]) {
+  if constexpr (!EMU) {
+    v[0] = finish1(nsum<double, false>(left, c[1], ym[0], yp[0], zm[0], zp[0]));
+    v[1] = finish1(nsum<double, false>(c[0], right, ym[1], yp[1], zm[1], zp[1]));
+  } else {
+    int f0 = 0, f1 = 0;
+    const double x0 = dadd_near(left, c[1], f0), y0 = dadd_near(ym[0], yp[0], f0), z0 = dadd_near(zm[0], zp[0], f0);
+    const double x1 = dadd_near(c[0], right, f1), y1 = dadd_near(ym[1], yp[1], f1), z1 = dadd_near(zm[1], zp[1], f1);
+    v[0] = finish1(__dadd_rn(__dadd_rn(x0, y0), z0));
+    v[1] = finish1(__dadd_rn(dadd_near(x1, y1, f1), z1));
+    if (!whole) f1 = 0;
+    if ((f0 | f1) < 0) {
+      if (f0 < 0) f0 = sum_far(left, c[1], ym[0], yp[0], zm[0], zp[0], false);
+      if (f1 < 0) f1 = sum_far(c[0], right, ym[1], yp[1], zm[1], zp[1], true);
+      if ((f0 | f1) < 0) {
+        v[0] = finish1(nsum<double, true>(left, c[1], ym[0], yp[0], zm[0], zp[0]));
+        v[1] = finish1(nsum<double, true>(c[0], right, ym[1], yp[1], zm[1], zp[1]));
+      }
+    }
+  }
 }
 template <bool EMU>
 __device__ __forceinline__ void update(const float (&c)[4], const float (&ym)[4], const float (&yp)[4], const float (&zm)[4],
-                                       const float (&zp)[4], float left, float right, float (&v)[4]) {
+                                       const float (&zp)[4], float left, float right, bool, float (&v)[4]) {
   float s[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
@@ -189,7 +210,7 @@ __device__ __forceinline__ void box_sweep(const BoxView& G, const ResBox& X, con
     V16<T>::load(src + off - G.plane, zm);
     V16<T>::load(src + off + G.plane, zp);
     const T left = src[off - 1], right = src[off + VEC];
-    update<EMU>(c, ym, yp, zm, zp, left, right, u);
+    update<EMU>(c, ym, yp, zm, zp, left, right, !(e & kTabPartial), u);
     if (!(e & kTabPartial)) {
       V16<T>::store(dst + off, u);
     } else {  // the rest of the vector is x halo and padding
