@@ -1059,9 +1059,13 @@ int compute_bnorm(jacobi_t* h, cudaStream_t s, bool new_state) {
   return JACOBI_OK;
 }
 
-int read_norms(jacobi_t* h, cudaStream_t s) {
+// The norms of every grid to the host; with_err also the error word, behind the
+// same synchronisation.
+int read_norms(jacobi_t* h, cudaStream_t s, bool with_err = false) {
   JGB_CUDA(cudaMemcpyAsync(h->h_norms, h->d_norms, h->plan.grids.size() * sizeof(GridNorm), cudaMemcpyDeviceToHost, s));
+  if (with_err) JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   JGB_CUDA(cudaStreamSynchronize(s));
+  if (with_err && *h->h_err != DEV_OK) return check_err_word(h, s);  // reads it again, clears it and reports
   return JACOBI_OK;
 }
 
@@ -1688,12 +1692,8 @@ int jacobi_solve(jacobi_t* h, double tol, int64_t max_iters, int64_t check_every
         rc = step_with_residual(h, s);
       }
       if (rc) return rc;
-      rc = read_norms(h, s);
+      rc = read_norms(h, s, h->path == JACOBI_PATH_PERSISTENT || h->res.ok);
       if (rc) return rc;
-      if (h->path == JACOBI_PATH_PERSISTENT || h->res.ok) {
-        rc = check_err_word(h, s);
-        if (rc) return rc;
-      }
       const bool stepped = done_k < max_iters;
       bool any_active = false;
       for (size_t g = 0; g < ng; ++g) {

@@ -31,13 +31,14 @@ template <> struct V16<double> {
 // Sum of the six neighbours in the stencil's order.  With EMU (FP64 states
 // inside the integer adder's domain) the three pair sums run on the integer
 // pipe and the two outer additions on the FP64 pipe: both pipes share the
-// work and the result is bit-identical.
+// work and the result is bit-identical (`third`: the sum of the first two pairs
+// is an integer one too).
 template <typename T, bool EMU>
-__device__ __forceinline__ T nsum(T xm, T xp, T ym, T yp, T zm, T zp) {
+__device__ __forceinline__ T nsum(T xm, T xp, T ym, T yp, T zm, T zp, bool third = false) {
   if (EMU) {
     const double sx = dadd_nn((double)xm, (double)xp), sy = dadd_nn((double)ym, (double)yp),
                  sz = dadd_nn((double)zm, (double)zp);
-    return (T)__dadd_rn(__dadd_rn(sx, sy), sz);
+    return (T)__dadd_rn(third ? dadd_nn(sx, sy) : __dadd_rn(sx, sy), sz);
   }
   return radd(radd(radd(xm, xp), radd(ym, yp)), radd(zm, zp));
 }
