@@ -56,13 +56,13 @@ __device__ __forceinline__ int64_t cell(const BlockDev& B, int64_t i, int64_t j,
 // nx elements long with pitch rx, so interior and slots take the same code; the
 // two x ghosts of an interior row are read beside it.  A block's rows are
 // split over nsub CTAs (state_split), a warp takes 32 / LPR rows at a time (LPR
-// lanes per row, 32 unless the block is narrower), and each lane keeps 4 rows x
-// 2 elements in flight.  With one CTA per block (before) a small grid left most
+// lanes per row, 32 unless the block is narrower), and each lane keeps eight
+// elements in flight.  With one CTA per block (before) a small grid left most
 // of the chip idle, and a batch paid that once per grid.  jacobi_set_state (with
 // its |b| and domain check) and jacobi_copy_out on the device, before -> now:
 // 64^3 FP64 in 32^3 blocks 130 -> 20 and 51 -> 13 us; 512^3 FP64 in 64^3 blocks
-// 2.69 -> 0.50 and 0.66 -> 0.36 ms; 768^3 FP32 7.8 -> 1.25 and 1.28 -> 0.99 ms; 256
-// FP32 grids of 16..192 set and read back 66 -> 9 ms.
+// 2.69 -> 0.50 and 0.66 -> 0.33 ms; 768^3 FP32 7.8 -> 1.25 and 1.28 -> 0.77 ms; 256
+// FP32 grids of 16..192 set and read back 66 -> 8.5 ms.
 // ---------------------------------------------------------------------------
 struct RowWalk {
   int lo, ey, r, r1, step, j, k, sj, sk, x, lpr;
@@ -245,34 +245,35 @@ __global__ void __launch_bounds__(kThreads) k_init(const BlockDev* __restrict__ 
   emu_flag(bad, norms, G.grid);
 }
 
-// CTAs [0, nb * nsub) install a padded array of one grid into its blocks
-// (parity p state and slots) and check its domain; the CTAs after them take one
-// work item each and write its |b|^2 partial, straight from the array.
+// CTAs [0, n_items) take one work item each and write its |b|^2 partial, straight
+// from a padded array of one grid (first, so that they do not trail); the
+// nb * nsub CTAs after them install the array into the grid's blocks (parity p
+// state and slots) and check its domain.
 template <typename T>
 __global__ void __launch_bounds__(kThreads, 4) k_scatter(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
-                                                      int32_t b0, int32_t nb, int32_t nsub, const T* __restrict__ src, int64_t NX,
-                                                      int64_t NY, int parity, const WorkItem* __restrict__ items, double* partials,
-                                                      GridNorm* norms) {
+                                                         int32_t b0, int32_t n_items, int32_t nsub, const T* __restrict__ src, int64_t NX,
+                                                         int64_t NY, int parity, const WorkItem* __restrict__ items, double* partials,
+                                                         GridNorm* norms) {
   __shared__ BlockDev B;
-  const int64_t px = NX + 2, py = NY + 2;
-  if ((int)blockIdx.x >= nb * nsub) {
-    const WorkItem w = items[blockIdx.x - nb * nsub];
+  const int64_t px = NX + 2, pp = px * (NY + 2);
+  if ((int)blockIdx.x < n_items) {
+    const WorkItem w = items[blockIdx.x];
     block_to_shared(B, blocks + w.block);
     const BlockGeom G = geom[w.block];
-    const T* base = src + ((int64_t)(G.oz + 1) * py + (G.oy + 1)) * px + (G.ox + 1);
-    const double acc = bnorm_item(B, w, ArrayGhost<T>{base, px, px * py});
+    const T* base = src + (int64_t)(G.oz + 1) * pp + (int64_t)(G.oy + 1) * px + (G.ox + 1);
+    const double acc = bnorm_item(B, w, ArrayGhost<T>{base, px, pp});
     __shared__ double red[kThreads / 32];
     const double s = block_sum<kThreads>(acc, red);
     if (threadIdx.x == 0) partials[w.slot] = s;
     return;
   }
-  const int b = b0 + blockIdx.x / nsub;
+  const int q = blockIdx.x - n_items, b = b0 + q / nsub;
   block_to_shared(B, blocks + b);
   const BlockGeom G = geom[b];
-  const T* __restrict__ base = src + ((int64_t)(G.oz + 1) * py + (G.oy + 1)) * px + (G.ox + 1);
+  const T* __restrict__ base = src + (int64_t)(G.oz + 1) * pp + (int64_t)(G.oy + 1) * px + (G.ox + 1);
   const int nx = B.nx;
   bool bad = false;
-  RowWalk W = row_walk(B, 1, blockIdx.x % nsub, nsub);
+  RowWalk W = row_walk(B, 1, q % nsub, nsub);
   while (W.r < W.r1) {
     constexpr int U = 4;
     const T* s[U];
@@ -282,7 +283,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(const BlockDev* __restr
     for (int u = 0; u < U; ++u) {
       const int j = W.j - 1, k = W.k - 1;
       d[u] = W.r < W.r1 ? ext_row<T>(B, parity, j, k) : nullptr;
-      s[u] = base + ((int64_t)k * py + j) * px;
+      s[u] = base + (int64_t)k * pp + (int64_t)j * px;
       const bool inside = d[u] && j >= 0 && j < B.ny && k >= 0 && k < B.nz;
       ge[u] = inside ? k * B.ry + j : -1;
       row_next(W);
@@ -331,58 +332,72 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(const BlockDev* __restr
   emu_flag(bad, norms, G.grid);
 }
 
-// Current iterate (parity p) back to an array of the whole grid: the interior,
-// or (padded) with the Dirichlet faces around it.
-template <typename T>
-__global__ void __launch_bounds__(kThreads, 4) k_gather(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
-                                                     int32_t b0, int32_t nsub, T* __restrict__ dst, int64_t NX, int64_t NY, int parity,
-                                                     int padded) {
-  __shared__ BlockDev B;
-  const int b = b0 + blockIdx.x / nsub;
-  block_to_shared(B, blocks + b);
-  const BlockGeom G = geom[b];
-  const int64_t px = NX + 2 * padded, py = NY + 2 * padded;
-  T* __restrict__ base = dst + ((int64_t)(G.oz + padded) * py + (G.oy + padded)) * px + (G.ox + padded);
+// Rows in flight of the gather: a lane holds U rows x E elements.  Rows are kept as
+// (k, j) in one word and their addresses derived twice, for the load and for the
+// store, which leaves the registers to the data: blocks of up to 32 columns take 8
+// rows x 1, wider ones 4 x 2 (512^3 FP32 in 32^3 blocks 572 -> 367 us, 768^3 in 64^3
+// blocks 992 -> 772 us against 4 x 2 with both pointers kept; the scatter, with its
+// domain check and x ghosts, spills so and keeps its pointers).
+__device__ __forceinline__ int row_pack(int j, int k) { return (k + 1) << 16 | (j + 1); }
+
+template <typename T, int U, int E>
+__device__ __forceinline__ void gather_rows(const BlockDev& B, RowWalk W, T* __restrict__ base, int64_t px, int64_t pp, int parity, int padded) {
   const int nx = B.nx;
-  RowWalk W = row_walk(B, padded, blockIdx.x % nsub, nsub);
   while (W.r < W.r1) {
-    constexpr int U = 4;
-    const T* s[U];
-    T* d[U];
+    int jk[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = W.j - padded, k = W.k - padded;
       bool take = W.r < W.r1;
       if (padded) {  // only Dirichlet faces lie on the padded boundary
-        if (j < 0) take = take && B.nbr[YM] < 0;
-        if (j >= B.ny) take = take && B.nbr[YP] < 0;
-        if (k < 0) take = take && B.nbr[ZM] < 0;
-        if (k >= B.nz) take = take && B.nbr[ZP] < 0;
+        const bool jo = j < 0 || j >= B.ny, ko = k < 0 || k >= B.nz;
+        if (jo) take = take && !ko && B.nbr[j < 0 ? YM : YP] < 0;
+        if (ko) take = take && !jo && B.nbr[k < 0 ? ZM : ZP] < 0;
+        if (take && !jo && !ko)
+          for (int g = W.x; g < 2; g += W.lpr)
+            if (B.nbr[g ? XP : XM] < 0)
+              base[(int64_t)k * pp + (int64_t)j * px + (g ? nx : -1)] = ((const T*)B.recv[g ? XP : XM][parity])[(int64_t)k * B.ry + j];
       }
-      s[u] = take ? ext_row<T>(B, parity, j, k) : nullptr;
-      d[u] = base + ((int64_t)k * py + j) * px;
-      if (padded && s[u] && j >= 0 && j < B.ny && k >= 0 && k < B.nz)
-        for (int g = W.x; g < 2; g += W.lpr)
-          if (B.nbr[g ? XP : XM] < 0) d[u][g ? nx : -1] = ((const T*)B.recv[g ? XP : XM][parity])[(int64_t)k * B.ry + j];
+      jk[u] = take ? row_pack(j, k) : -1;
       row_next(W);
     }
-    for (int i = W.x; i < nx; i += 2 * W.lpr) {
-      T v[U][2];
-      const bool two = i + W.lpr < nx;
+    for (int i = W.x; i < nx; i += E * W.lpr) {
+      T v[U][E];
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (s[u]) {
-          v[u][0] = s[u][i];
-          if (two) v[u][1] = s[u][i + W.lpr];
-        }
+      for (int u = 0; u < U; ++u) {
+        if (jk[u] < 0) continue;
+        const T* s = ext_row<T>(B, parity, (jk[u] & 0xFFFF) - 1, (jk[u] >> 16) - 1);
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (s[u]) {
-          d[u][i] = v[u][0];
-          if (two) d[u][i + W.lpr] = v[u][1];
-        }
+        for (int e = 0; e < E; ++e)
+          if (i + e * W.lpr < nx) v[u][e] = s[i + e * W.lpr];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (jk[u] < 0) continue;
+        T* d = base + ((int64_t)((jk[u] >> 16) - 1) * pp + (int64_t)((jk[u] & 0xFFFF) - 1) * px);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (i + e * W.lpr < nx) d[i + e * W.lpr] = v[u][e];
+      }
     }
   }
+}
+
+// Current iterate (parity p) back to an array of the whole grid: the interior,
+// or (padded) with the Dirichlet faces around it.
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 4) k_gather(const BlockDev* __restrict__ blocks, const BlockGeom* __restrict__ geom,
+                                                        int32_t b0, int32_t nsub, T* __restrict__ dst, int64_t NX, int64_t NY, int parity,
+                                                        int padded) {
+  __shared__ BlockDev B;
+  const int b = b0 + blockIdx.x / nsub;
+  block_to_shared(B, blocks + b);
+  const BlockGeom G = geom[b];
+  const int64_t px = NX + 2 * padded, pp = px * (NY + 2 * padded);
+  T* __restrict__ base = dst + (int64_t)(G.oz + padded) * pp + (int64_t)(G.oy + padded) * px + (G.ox + padded);
+  const RowWalk W = row_walk(B, padded, blockIdx.x % nsub, nsub);
+  if (B.nx <= 32) gather_rows<T, 8, 1>(B, W, base, px, pp, parity, padded);
+  else gather_rows<T, 4, 2>(B, W, base, px, pp, parity, padded);
 }
 
 // |b|^2 partials of work items from the receive slots.
@@ -620,9 +635,9 @@ cudaError_t launch_scatter(const BlockDev* blocks, const BlockGeom* geom, int32_
   const int nsub = state_split(nb, max_rows);
   const unsigned grid = (unsigned)((int64_t)nb * nsub + n_items);
   if (dtype == 0)
-    k_scatter<double><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nb, nsub, (const double*)src, NX, NY, parity, items, partials, norms);
+    k_scatter<double><<<grid, kThreads, 0, s>>>(blocks, geom, b0, n_items, nsub, (const double*)src, NX, NY, parity, items, partials, norms);
   else
-    k_scatter<float><<<grid, kThreads, 0, s>>>(blocks, geom, b0, nb, nsub, (const float*)src, NX, NY, parity, items, partials, norms);
+    k_scatter<float><<<grid, kThreads, 0, s>>>(blocks, geom, b0, n_items, nsub, (const float*)src, NX, NY, parity, items, partials, norms);
   return cudaGetLastError();
 }
 
