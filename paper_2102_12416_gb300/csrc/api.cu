@@ -983,13 +983,18 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   a.ctl = R.d_ctl;
   a.err = h->d_err;
   a.wait_ns = h->wait_ns;
-  a.it0 = it0;
-  a.n_iters = n;
   a.n_boxes = R.n_boxes;
   a.smem = R.smem;
   a.dtype = h->plan.dtype;
   a.emu = h->fp64_emu;
-  JGB_CUDA(launch_resident(a, s));
+  // A launch holds every SM until it ends: long calls are split, at some 30 to 150
+  // ms each, so that other streams get their turn.
+  for (int64_t done = 0; done < n;) {
+    a.it0 = it0 + done;
+    a.n_iters = std::min<int64_t>(n - done, 16384);
+    JGB_CUDA(launch_resident(a, s));
+    done += a.n_iters;
+  }
   return JACOBI_OK;
 }
 

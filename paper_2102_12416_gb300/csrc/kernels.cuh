@@ -223,7 +223,7 @@ struct ResLaunch {
   const GridDev* grids;
   const GridNorm* norms;  // per-grid emu_bad flags
   uint4* packets;
-  uint32_t* ctl;          // [0] next sequence number, [1] CTAs that have finished
+  uint32_t* ctl;          // [0] next sequence number, [1] CTAs that have finished, [2] that have started
   uint32_t* err;
   uint64_t wait_ns;
   int64_t it0, n_iters;

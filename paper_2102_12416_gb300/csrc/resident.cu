@@ -27,7 +27,10 @@
 // surface of iteration t + 2 only after it has received its neighbour's of t + 1,
 // which the neighbour sent after all its threads had read t: the buffer is free.
 // Sequence numbers continue from launch to launch (ctl[0], advanced by the last
-// CTA to finish), so nothing is cleared between launches.  Waits are bounded.
+// CTA to finish), so nothing is cleared between launches.  Waits are bounded; the
+// limit counts from when all CTAs have started (ctl[2], looked at only when a wait
+// runs out), which other streams' kernels may delay.  (A meeting of all CTAs before
+// the second iteration instead cost 3 us a call.)
 #include <vector>
 
 #include "kernels.cuh"
@@ -139,6 +142,8 @@ __device__ __forceinline__ void update(const float (&c)[4], const float (&ym)[4]
   finish_vec(s, v);
 }
 
+constexpr uint64_t kResStartNs = 30000000000ull;
+
 // Threads per CTA: as many as the registers of an update allow (FP32 64, FP64
 // 85 per thread), since the sweep is latency-bound with fewer warps: one box of
 // 4096 FP32 points took 1.9 us with 512 threads, 1.3 with 1024.
@@ -236,6 +241,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
   __syncthreads();
   for (int q = tid; q < (int)(sizeof(ResGrid) / 4); q += NT) ((uint32_t*)&R)[q] = ((const uint32_t*)(a.rgrids + X.rgrid))[q];
   const uint32_t base = *(volatile const uint32_t*)a.ctl;  // sequence number of the launch's first state
+  if (tid == 0) atomicAdd(a.ctl + 2, 1u);                  // this CTA has started
   __syncthreads();
   const GridDev GD = a.grids[R.grid];
   if (GD.active) {
@@ -352,7 +358,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
         for (int h0 = tid; ok && (h0 < X.n_vec || h0 < X.n_one); h0 += 2 * NT) {
           // entries h0 and h0 + NT of the vectors; x values go in steps of NT, two rounds per step of 2 NT
           bool want[4] = {h0 < X.n_vec, h0 + NT < X.n_vec, h0 < X.n_one, h0 + NT < X.n_one};
-          uint64_t t0 = 0;
+          uint64_t t0 = 0, first = 0;
           for (uint32_t n = 0;; ++n) {
             uint32_t w[4][4];
             bool got[4];
@@ -375,8 +381,16 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
               }
             if (!(want[0] || want[1] || want[2] || want[3])) break;
             if ((n & 63u) != 63u) continue;
-            if (t0 == 0) t0 = globaltimer_ns();
-            if (ld_volatile_u32(a.err) != DEV_OK || globaltimer_ns() - t0 > a.wait_ns || n > (1u << 28)) {
+            const uint64_t now = globaltimer_ns();
+            if (t0 == 0) t0 = first = now;
+            bool stop = ld_volatile_u32(a.err) != DEV_OK || n > (1u << 30);
+            if (now - t0 > a.wait_ns) {
+              // the limit counts from when every CTA has started: other streams'
+              // kernels may still hold some of the SMs
+              if (ld_acquire_u32(a.ctl + 2) < gridDim.x && now - first < kResStartNs) t0 = now;
+              else stop = true;
+            }
+            if (stop) {
               atomicCAS(a.err, (uint32_t)DEV_OK, (uint32_t)DEV_TIMEOUT);
               ok = false;
               break;
@@ -421,6 +435,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
   // the last CTA advances the sequence numbers for the next launch
   if (tid == 0 && atomicAdd(a.ctl + 1, 1u) == gridDim.x - 1) {
     a.ctl[1] = 0u;
+    a.ctl[2] = 0u;
     a.ctl[0] = base + (uint32_t)a.n_iters;
   }
 }

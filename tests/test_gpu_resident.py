@@ -64,3 +64,22 @@ def test_resident_batch_solve_freezes_grids(dtype, monkeypatch):
             got.append((res, [s.copy_out(g) for g in range(4)]))
     assert got[0][0] == got[1][0] and len(set(got[0][0][0])) > 1
     assert all(np.array_equal(a, b) for a, b in zip(got[0][1], got[1][1]))
+
+
+def test_resident_on_two_streams_and_long_calls():
+    """Two handles whose resident launches overlap on the GPU, each in more than one launch per call (16384 iterations at most)."""
+    import torch
+
+    import paper_2102_12416_gb300 as jg
+    grid, n = (20, 17, 19), 20011
+    u = [J.initial_grid(*grid, bc="uniform", bc_seed=q, interior="uniform", interior_seed=q + 9, dtype=np.float32) for q in (1, 2)]
+    streams = [torch.cuda.Stream() for _ in u]
+    hs = [jg.Jacobi3D(grid, ("shape", (8, 8, 8)), "f32", path="graph", stream=s) for s in streams]
+    for h, x in zip(hs, u):
+        h.set_state(x)
+    for h in hs:
+        h.step(n)
+    for h, x in zip(hs, u):
+        h.sync()
+        assert np.array_equal(h.copy_out(), J.interior_of(oracle.jacobi(x, n)))
+        h.close()
