@@ -259,7 +259,9 @@ int jacobi_workspace_bytes_batch(int64_t n_grids, const jacobi_dim3* grids,
 /* Create a solver for one grid.  `init` may be NULL (linear boundary, zero
  * interior).  `workspace` may be NULL (the library allocates and frees it)
  * or a device buffer of at least jacobi_workspace_bytes() bytes, 256-byte
- * aligned, owned by the caller.  The initial state is written by a kernel on
+ * aligned, owned by the caller (beside it the library allocates the resident
+ * path's tables, a few MB, for grids that path takes, and staging buffers when a
+ * call first needs them).  The initial state is written by a kernel on
  * `stream`; the call returns without waiting for it. */
 int jacobi_create(jacobi_dim3 grid, jacobi_split split, jacobi_dtype dtype,
                   const jacobi_init* init, void* workspace, size_t ws_bytes, void* stream,
@@ -383,15 +385,16 @@ int jacobi_sync(jacobi_t* h, void* stream);
  * Dirichlet boundary).  Synchronises the stream. */
 int jacobi_read_face(jacobi_t* h, int64_t block, int32_t face, void* dst, void* stream);
 
-/* Test support for the integer-pipe FP64 adder: out[i] = a[i] + b[i] (device
+/* Test support for the integer-pipe FP64 adders: out[i] = a[i] + b[i] (device
  * arrays of n doubles) computed by the integer-pipe routine the FP64 step
- * kernels use for the neighbour pair sums and the FP32 residual for the pair
- * sums of its widened values.  For a[i], b[i] >= 0 with
+ * kernels use for the neighbour pair sums, or NaN where the shorter routine for
+ * close exponents (resident kernel, allocation-free residual) reaches and
+ * differs from it.  For a[i], b[i] >= 0 with
  * exponent field < 2040 the result is the IEEE-754 round-to-nearest-even sum
  * bit for bit; other inputs give unspecified values (the step kernels never
  * pass them: a device check keeps such grids on the FP64 pipe).  Setting the
  * environment variable JACOBI_FP64_EMU=0 before jacobi_create keeps every
- * FP64 add on the FP64 pipe.  Asynchronous. */
+ * FP64 add of the step kernels on the FP64 pipe.  Asynchronous. */
 int jacobi_selftest_dadd(const double* a, const double* b, int64_t n, double* out, void* stream);
 
 /* Test support for the FP32 residual's exact binary32 -> binary64 widening on
@@ -402,10 +405,11 @@ int jacobi_selftest_dadd(const double* a, const double* b, int64_t n, double* ou
 int jacobi_selftest_widen(uint64_t* mismatches, void* stream);
 
 /* Test support for the FP32 update's division: u' = RN(s / 6) is computed as
- * RN(s * zh + RN(s * zl)) with zh = RN(1/6), zl = RN(1/6 - zh) (a method of
+ * RN(s * zh + RN(s * zl)) with zh the largest float below 1/6 and zl =
+ * RN(1/6 - zh) (a method of
  * Brisebarre, Muller and Raina for division by a constant; the paper prints no
- * stencil, see the arithmetic note at the top of this file), with the
- * division instruction sequence for the inputs outside that form's proven
+ * stencil, see the arithmetic note at the top of this file), with integer
+ * arithmetic for the tiny inputs outside that form's proven
  * domain.  Runs all 2^32 binary32 bit patterns through it on the device and
  * writes to *mismatches (host) how many differ bit for bit from the division
  * instruction sequence (NaN inputs must give a NaN).  Expected 0.

@@ -992,7 +992,15 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   for (int64_t done = 0; done < n;) {
     a.it0 = it0 + done;
     a.n_iters = std::min<int64_t>(n - done, 16384);
-    JGB_CUDA(launch_resident(a, s));
+    const cudaError_t e = launch_resident(a, s);
+    if (e != cudaSuccess && done == 0) {
+      // refused before anything ran (say, fewer SMs than the device reports are
+      // open to this process): the handle keeps to the other kernels
+      cudaGetLastError();
+      h->res.ok = false;
+      return JACOBI_EAGAIN;
+    }
+    JGB_CUDA(e);
     done += a.n_iters;
   }
   return JACOBI_OK;
@@ -1008,9 +1016,8 @@ int do_step(jacobi_t* h, int64_t n, cudaStream_t s) {
   }
   if (resident_applies(h, n, s)) {
     rc = step_resident(h, h->iter, n, s);
-    if (rc) return rc;
-    h->iter += n;
-    return JACOBI_OK;
+    if (rc == JACOBI_OK) h->iter += n;
+    if (rc != JACOBI_EAGAIN) return rc;
   }
   switch (h->path) {
     case JACOBI_PATH_FUSED: rc = step_fused_direct(h, h->iter, n, s); break;
@@ -1463,6 +1470,9 @@ static int autotune_search(jacobi_t* h, int64_t iters_per_trial, void* stream, j
     int rc = jacobi_create_batch((int64_t)grids.size(), grids.data(), splits.data(), (jacobi_dtype)P.dtype,
                                  inits.data(), nullptr, 0, stream, &t);
     if (rc) return rc;
+    // The candidates are the kernels that path, depth and shape choose between;
+    // calls that the resident kernel takes do not depend on them.
+    t->res.allowed = t->res.ok = false;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);

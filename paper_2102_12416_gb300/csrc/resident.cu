@@ -31,6 +31,7 @@
 // limit counts from when all CTAs have started (ctl[2], looked at only when a wait
 // runs out), which other streams' kernels may delay.  (A meeting of all CTAs before
 // the second iteration instead cost 3 us a call.)
+#include <atomic>
 #include <vector>
 
 #include "kernels.cuh"
@@ -440,9 +441,16 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
   }
 }
 
+// The shared-memory opt-in, once per device.
 template <typename T>
 cudaError_t resident_attr() {
-  static const cudaError_t e = cudaFuncSetAttribute(k_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
+  static std::atomic<uint64_t> done{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  const uint64_t bit = 1ull << (dev & 63);
+  if (e != cudaSuccess || (dev < 64 && (done.load() & bit))) return e;
+  e = cudaFuncSetAttribute(k_resident<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
+  if (e == cudaSuccess && dev < 64) done.fetch_or(bit);
   return e;
 }
 
