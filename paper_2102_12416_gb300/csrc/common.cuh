@@ -167,12 +167,15 @@ __device__ __forceinline__ int exp_far(double a, double b, int reach) {
   const bool zero = __double_as_longlong(a) == 0 || __double_as_longlong(b) == 0;
   return (abs(ea - eb) > reach && !zero) ? -1 : 0;
 }
-__device__ __forceinline__ double larger_hi(double a, double b) { return __double2hiint(a) >= __double2hiint(b) ? a : b; }
+// The larger operand (of values with a clear sign bit): all 64 bits count, since
+// 0 and the subnormals below 2^-1042 have the same high word, and a pair of them
+// is not zero.
+__device__ __forceinline__ double larger(double a, double b) { return __double_as_longlong(a) >= __double_as_longlong(b) ? a : b; }
 // The same for a point's three pair sums and, with `third`, the sum of the first
 // two (it stays within reach if the pairs are one binade closer).
 __device__ __forceinline__ int sum_far(double xm, double xp, double ym, double yp, double zm, double zp, bool third) {
   int f = exp_far(xm, xp, 10) | exp_far(ym, yp, 10) | exp_far(zm, zp, 10);
-  if (third) f |= exp_far(larger_hi(xm, xp), larger_hi(ym, yp), 9);
+  if (third) f |= exp_far(larger(xm, xp), larger(ym, yp), 9);
   return f;
 }
 
