@@ -329,12 +329,7 @@ __device__ __forceinline__ float two_sum_err(float a, float b, float t) {
 // taken in FP64 (8 operations per point with r's square) but in FP32 together
 // with the exact rounding error of each of its five additions, of 6u and of the
 // difference; only the last addition d + e and the square are left to FP64.
-// The error terms are multiples of the smallest neighbour's ulp and at most
-// half an ulp of s: their FP32 sum e is exact while the nonzero neighbours
-// (and u) span up to 2^19, and beyond that off by at most 2^-24 of itself,
-// 2^-46 of s.  Where the FP64 sums are exact too (a span of up to 2^26) r is
-// the same number.  False when an operation overflowed, or on a NaN: the caller
-// then takes the sums in FP64.
+// False when an operation overflowed, or on a NaN.
 __device__ __forceinline__ bool resid_split(float xm, float xp, float ym, float yp, float zm, float zp, float c, float& d,
                                             float& e) {
   const float tx = __fadd_rn(xm, xp), ty = __fadd_rn(ym, yp), tz = __fadd_rn(zm, zp);
@@ -347,8 +342,43 @@ __device__ __forceinline__ bool resid_split(float xm, float xp, float ym, float 
   e = __fadd_rn(__fadd_rn(ea, eb), ec);
   return fabsf(__fadd_rn(d, e)) <= 0x1.fffffep+127f;
 }
-// The same residual with every sum in FP64 (a call: it is rarely taken, and its
-// temporaries would cost the callers registers).
+// Whether that r is the number that the FP64 sums give, bit for bit: the form is
+// taken only where both are exact.  Let the nonzero neighbours and u have
+// exponents between f and F (subnormals count as the smallest normal exponent).
+// The seven error terms are multiples of 2^(f - 23) and, as half ulps of sums of up
+// to 12 operands, at most (1 + 1 + 1 + 2 + 4 + 4 + 8) * 2^(F - 23) together, so with
+// F - f <= 19 every FP32 sum of them is below 2^24 * 2^(f - 23) and exact; r needs
+// 47 bits.  Elsewhere the sums are taken in FP64.
+constexpr uint32_t kSplitSpan = 19;
+// The magnitudes of a set of operands: the largest, and the smallest but zero (its
+// bits doubled, less one, so that zeros wrap to the top).
+struct Magnitudes {
+  float top = 0.0f;
+  uint32_t low = ~0u;
+  __device__ __forceinline__ void add(float v) {
+    top = fmaxf(top, fabsf(v));
+    low = min(low, 2u * __float_as_uint(v) - 1u);
+  }
+  template <int N>
+  __device__ __forceinline__ void add(const float (&v)[N]) {  // one after another: rows that points share are looked at once
+    Magnitudes m;
+#pragma unroll
+    for (int q = 0; q < N; ++q) m.add(v[q]);
+    top = fmaxf(top, m.top);
+    low = min(low, m.low);
+  }
+  __device__ __forceinline__ bool split_exact() const {
+    return (__float_as_uint(top) >> 23) <= max((low + 1u) >> 24, 1u) + kSplitSpan;
+  }
+};
+// A point's operands, and its residual with every sum in FP64 (calls: both are
+// rarely wanted, and their temporaries would cost the callers registers).
+static __device__ __noinline__ bool point_exact(float xm, float xp, float ym, float yp, float zm, float zp, float c) {
+  const float v[7] = {xm, xp, ym, yp, zm, zp, c};
+  Magnitudes m;
+  m.add(v);
+  return m.split_exact();
+}
 static __device__ __noinline__ double resid_f64(float xm, float xp, float ym, float yp, float zm, float zp, float c) {
   const double s = __dadd_rn(__dadd_rn(__dadd_rn(widen_f32(xm), widen_f32(xp)), __dadd_rn(widen_f32(ym), widen_f32(yp))),
                              __dadd_rn(widen_f32(zm), widen_f32(zp)));

@@ -31,7 +31,8 @@ static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxPlanes];
 // r = s - 6u of one point.  FP64: four of the five sums on the integer pipe when
 // all lanes' neighbours are inside the adders' domain (the same rounded sums, by
 // dadd_near, or dadd_nn where some lane's are out of its reach; the last sum, 6u,
-// the difference and the square stay on the FP64 pipe).  FP32: resid_split.
+// the difference and the square stay on the FP64 pipe).  FP32: resid_split where the
+// operands' magnitudes show it to be exact.
 __device__ __forceinline__ double noalloc_r(double xm, double xp, double ym, double yp, double zm, double zp, double c, bool use) {
   const uint32_t hi = max(max(max((uint32_t)__double2hiint(xm), (uint32_t)__double2hiint(xp)),
                               max((uint32_t)__double2hiint(ym), (uint32_t)__double2hiint(yp))),
@@ -52,8 +53,11 @@ __device__ __forceinline__ double noalloc_r(double xm, double xp, double ym, dou
   return __dsub_rn(__dadd_rn(sxy, sz), __dmul_rn(6.0, c));
 }
 __device__ __forceinline__ double noalloc_r(float xm, float xp, float ym, float yp, float zm, float zp, float c, bool) {
+  const float v[7] = {xm, xp, ym, yp, zm, zp, c};
+  Magnitudes m;
+  m.add(v);
   float d, e;
-  if (resid_split(xm, xp, ym, yp, zm, zp, c, d, e)) return __dadd_rn(widen_f32(d), widen_f32(e));
+  if (resid_split(xm, xp, ym, yp, zm, zp, c, d, e) && m.split_exact()) return __dadd_rn(widen_f32(d), widen_f32(e));
   return resid_f64(xm, xp, ym, yp, zm, zp, c);
 }
 

@@ -75,13 +75,16 @@ __device__ __forceinline__ bool mbar_ready(uint64_t* b, uint32_t parity, uint32_
   return mbar_test(b, parity) || mbar_wait(b, parity, err, limit_ns);
 }
 
-// Residual contributions r^2 of N neighbouring points, r = s - 6u in FP64 from
-// the state's values, added to acc in order; points with use[q] false add
+// Residual contributions r^2 of N neighbouring points of a row, r = s - 6u in FP64
+// from the state's values, added to acc in order; points with use[q] false add
 // nothing.  FP64: s is the stencil's own sum.  FP32: resid_split, FP64 sums only
-// where it cannot (one branch per vector): same-box, jacobi_residual at 768^3 in
-// 64^3 blocks 5.87 -> 2.08 ms, at 512^3 1.79 -> 0.67 ms, 32 served solves 550 ->
-// 540 ms, against sums of integer-widened values on the FP64 and integer pipes;
-// the norms are the same, and the step-and-residual kernels no longer spill.
+// where it is not exact (one branch per vector).  jacobi_residual at 768^3 in 64^3
+// blocks 2.11 ms, at 512^3 0.67 ms (5.87 and 1.79 with all sums in FP64, of
+// integer-widened values; the norms are the same).  The look at the operands' span
+// is 12 % of it, taken once per vector (22 operands): at each point, 17 %.  It finds a
+// vector on the front of a zero interior too wide (its points, less so, are looked
+// at one by one): 2.30 ms at 768^3 after 40 iterations, 2.66 if they go to the
+// whole FP64 residual at once.
 template <int N>
 __device__ __forceinline__ void resid_add(double& acc, const double (&)[N], const double (&)[N], const double (&)[N],
                                           const double (&)[N], const double (&)[N], const double (&)[N], const double (&s)[N],
@@ -97,6 +100,14 @@ __device__ __forceinline__ void resid_add(double& acc, const float (&xm)[N], con
                                           const float (&yp)[N], const float (&zm)[N], const float (&zp)[N], const float (&)[N],
                                           const float (&c)[N], const bool (&use)[N]) {
   double a = acc;
+  Magnitudes m;
+  m.add(c);
+  m.add(ym);
+  m.add(yp);
+  m.add(zm);
+  m.add(zp);
+  m.add(xm[0]);  // (the other x neighbours are c's)
+  m.add(xp[N - 1]);
   bool ok = true;
 #pragma unroll
   for (int q = 0; q < N; ++q) {
@@ -105,6 +116,11 @@ __device__ __forceinline__ void resid_add(double& acc, const float (&xm)[N], con
     double r = __dadd_rn(widen_f32(d), widen_f32(e));
     if (!use[q]) r = 0.0;
     a = fma(r, r, a);
+  }
+  if (!m.split_exact()) {  // some point may still be
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (use[q]) ok = point_exact(xm[q], xp[q], ym[q], yp[q], zm[q], zp[q], c[q]) && ok;
   }
   if (!ok) {
     a = acc;

@@ -1,5 +1,6 @@
 """The device arithmetic of csrc/common.cuh, compiled for the host (its intrinsics spelled as plain IEEE operations) and compared with
-FP64 sums where it can go wrong: six neighbours of any mixture of zeros, subnormals and normal values."""
+FP64 sums where it can go wrong: six neighbours of any mixture of zeros, subnormals and normal values; the residual of FP32 states over
+spans, signs and cancelling neighbours of all kinds."""
 import ctypes
 import os
 import subprocess
@@ -19,7 +20,7 @@ SHIM = r"""
 #define __host__
 #define __forceinline__ inline
 #define __noinline__
-using std::max; using std::min;
+using std::max; using std::min; using std::fabs;
 template <class A, class B> static inline A bits(B b) { A a; static_assert(sizeof(a) == sizeof(b), ""); memcpy(&a, &b, sizeof a); return a; }
 static inline double __dadd_rn(double a, double b) { return a + b; }
 static inline double __dsub_rn(double a, double b) { return a - b; }
@@ -60,6 +61,17 @@ void near_sums(const double* v, int64_t n, double* out) {
     else out[i] = s + z;
   }
 }
+// The residual of FP32 values; counts the points that the split form takes.
+int64_t resid32(const float* v, int64_t n, double* out) {
+  int64_t split = 0;
+  for (int64_t i = 0; i < n; ++i, v += 7) {
+    float d, e;
+    const bool ok = resid_split(v[0], v[1], v[2], v[3], v[4], v[5], v[6], d, e) && point_exact(v[0], v[1], v[2], v[3], v[4], v[5], v[6]);
+    split += ok;
+    out[i] = ok ? widen_f32(d) + widen_f32(e) : resid_f64(v[0], v[1], v[2], v[3], v[4], v[5], v[6]);
+  }
+  return split;
+}
 }
 """
 
@@ -76,7 +88,8 @@ def lib(tmp_path_factory):
 
 
 def _call(fn, v, out):
-    fn(ctypes.c_void_p(v.ctypes.data), ctypes.c_int64(len(v)), *(ctypes.c_void_p(o.ctypes.data) for o in out))
+    fn.restype = ctypes.c_int64
+    return fn(ctypes.c_void_p(v.ctypes.data), ctypes.c_int64(len(v)), *(ctypes.c_void_p(o.ctypes.data) for o in out))
 
 
 def _mixed64(n, seed):
@@ -102,3 +115,40 @@ def test_short_adder_far_operands(lib):
         want = ((v[:, 0] + v[:, 1]) + (v[:, 2] + v[:, 3])) + (v[:, 4] + v[:, 5])
         bad = np.nonzero(got.view(np.int64) != want.view(np.int64))[0]
         assert len(bad) == 0, (len(bad), [float(x).hex() for x in v[bad[0]]])
+
+
+def _states32(n):
+    """(what, rows of six neighbours and u, share that the split form must take)"""
+    r = np.random.default_rng(5)
+    one = r.uniform(0.5, 1.0, (n, 7))
+    sign = r.choice([-1.0, 1.0], (n, 7))
+    wide = 2.0 ** r.integers(-26, 1, (n, 7))  # spans around 2^19, where the split form ends
+    cancel = one * 2.0 ** r.integers(-40, -20, (n, 7))
+    k = r.integers(0, 3, n) * 2
+    cancel[np.arange(n), k] = one[:, 0]
+    cancel[np.arange(n), k + 1] = -one[:, 0]
+    u = one[:, :6].sum(1) / 6.0
+    near = one.copy()
+    near[:, 6] = np.float32(u) * (1 + 2.0 ** -23 * r.integers(-3, 4, n))  # near convergence: |r| far below the sums
+    sparse = np.where(r.uniform(size=(n, 7)) < 0.4, 0.0, one * sign)
+    return [("plain", one, 1.0), ("signed", one * sign, 1.0), ("near", near, 1.0), ("zeros", sparse, 1.0), ("wide", one * wide, 0.05),
+            ("wide signed", one * wide * sign, 0.05), ("cancel", cancel, 0.0), ("smooth", 3.0 + 1e-3 * one, 1.0),
+            ("exponents", one * sign * 2.0 ** r.integers(-149, 128, (n, 7)), 0.0), ("subnormal", one * sign * 2.0 ** -135, 1.0),
+            ("overflow", np.where(r.uniform(size=(n, 7)) < 0.3, 3.0e38, one) * sign, 0.0),
+            ("inf", np.where(r.uniform(size=(n, 7)) < 0.1, np.inf, one), 0.0), ("nan", np.where(r.uniform(size=(n, 7)) < 0.1, np.nan, one), 0.0)]
+
+
+def test_fp32_residual_is_that_of_fp64_sums(lib):
+    """r of every point equals the FP64 sums of the widened values: where the split form is taken every term is exact, elsewhere the
+    FP64 sums themselves are.  The split form takes all points of ordinary states."""
+    for what, rows, share in _states32(1 << 18):
+        with np.errstate(over="ignore"):
+            v = np.ascontiguousarray(rows.astype(np.float32))
+        got = np.empty(len(v))
+        split = _call(lib.resid32, v, [got])
+        w = v.astype(np.float64)
+        with np.errstate(invalid="ignore"):
+            want = (((w[:, 0] + w[:, 1]) + (w[:, 2] + w[:, 3])) + (w[:, 4] + w[:, 5])) - 6.0 * w[:, 6]
+        bad = np.nonzero((got != want) & ~(np.isnan(got) & np.isnan(want)))[0]
+        assert len(bad) == 0, (what, len(bad), [float(x).hex() for x in v[bad[0]]], got[bad[0]], want[bad[0]])
+        assert split >= share * len(v), (what, split)
