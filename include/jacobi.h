@@ -214,7 +214,7 @@ typedef struct {
                             blocks with padded (ragged) rows; [7] unused */
   int64_t zchunk;        /* work-item shape (see jacobi_set_shape): planes per item */
   int32_t cw_cap;        /*   and the consumer-warp cap of streaming CTAs         */
-  int32_t pad2_;
+  int32_t resident_launches; /* launches of the resident kernel so far (see jacobi_path) */
 } jacobi_info_t;
 
 /* Outcome of jacobi_autotune. */

@@ -70,7 +70,7 @@ class jacobi_info_t(ctypes.Structure):
                 ("iteration", c_int64), ("dtype", c_int32), ("path", c_int32),
                 ("halo_bytes_per_iter", c_int64), ("workspace_bytes", c_size_t), ("stages", c_int32),
                 ("item_kinds", c_int32), ("fp64_int_adds", c_int32), ("pad_", c_int32),
-                ("kind_items", c_int32 * 8), ("zchunk", c_int64), ("cw_cap", c_int32), ("pad2_", c_int32)]
+                ("kind_items", c_int32 * 8), ("zchunk", c_int64), ("cw_cap", c_int32), ("resident_launches", c_int32)]
 
 
 class jacobi_tune_result(ctypes.Structure):

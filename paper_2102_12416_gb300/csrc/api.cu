@@ -1001,6 +1001,7 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
       return JACOBI_EAGAIN;
     }
     JGB_CUDA(e);
+    h->res.launches += 1;
     done += a.n_iters;
   }
   return JACOBI_OK;
@@ -1385,7 +1386,7 @@ int jacobi_info(const jacobi_t* h, jacobi_info_t* out) {
   for (int k = 0; k < 8; ++k) out->kind_items[k] = k < kItemKinds ? h->kind_off[k + 1] - h->kind_off[k] : 0;
   out->zchunk = h->plan.zchunk;
   out->cw_cap = h->plan.cw_cap;
-  out->pad2_ = 0;
+  out->resident_launches = (int32_t)h->res.launches;
   return JACOBI_OK;
 }
 

@@ -122,6 +122,7 @@ struct Resident {
   bool ok = false;       // the active grids fit
   int n_boxes = 0, smem = 0;
   int64_t min_iters = 0; // shortest call it takes
+  int64_t launches = 0;  // so far, for jacobi_info
   char* with_ws = nullptr;
   char* own = nullptr;
   size_t own_bytes = 0;
