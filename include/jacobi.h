@@ -136,7 +136,11 @@ typedef struct { int32_t mode; int32_t pad_; int64_t x, y, z; } jacobi_split;
  * small enough to stay on chip (together about 1.3 M FP64 or 2.6 M FP32 points)
  * runs as one cooperative launch of the resident kernel instead: boxes of the
  * grids stay in shared memory and exchange their surfaces every iteration
- * through packets in device memory (bounded waits, reported as on PERSISTENT);
+ * through packets in device memory.  Its waits are bounded: when one expires,
+ * the next call that waits for the handle's work (jacobi_sync,
+ * jacobi_residual, jacobi_solve, jacobi_step_timed, jacobi_read_face,
+ * jacobi_copy_out to the host) returns JACOBI_ETIMEDOUT, and the state is
+ * unspecified until jacobi_set_state;
  * state and receive slots of the last iteration are written back.  The
  * environment variable JACOBI_RESIDENT=0 at creation turns it off, as does a
  * set JACOBI_PERSIST_WS; a stream under capture does not use it.
@@ -337,7 +341,8 @@ int jacobi_set_state(jacobi_t* h, int64_t grid, const void* src, int32_t src_on_
 
 /* Copy grid `grid`'s current iterate out in the interior or padded layout
  * (dtype of the handle).  dst_on_device = 0 (host; the call synchronises the
- * stream) or 1 (device; asynchronous). */
+ * stream and reports a resident step that gave up) or 1 (device; asynchronous:
+ * jacobi_sync reports it). */
 int jacobi_copy_out(jacobi_t* h, int64_t grid, void* dst, int32_t dst_on_device, int32_t layout,
                     void* stream);
 
@@ -374,7 +379,7 @@ int jacobi_solve(jacobi_t* h, double tol, int64_t max_iters, int64_t check_every
                  void* stream);
 
 /* Synchronise `stream` and report the first device-side failure of the
- * handle's persistent steps (JACOBI_ETIMEDOUT when a bounded neighbour wait
+ * handle's persistent or resident steps (JACOBI_ETIMEDOUT when a bounded neighbour wait
  * expired) or JACOBI_OK; clears it. */
 int jacobi_sync(jacobi_t* h, void* stream);
 
@@ -428,6 +433,12 @@ int jacobi_pipe_rates(double* fp64_adds_per_s, double* int_adds_per_s, void* str
  * bounded waits expire and jacobi_sync reports JACOBI_ETIMEDOUT.  block = -1
  * clears the injection. */
 int jacobi_debug_drop_block(jacobi_t* h, int64_t block);
+
+/* The same for the resident kernel: its next launches are those of a box
+ * `what` >= 0 that sends nothing, so that the boxes beside it give up after the
+ * wait limit, or (what = -2) ask for more shared memory than there is, so that
+ * the runtime refuses them and the other kernels run.  what = -1 clears it. */
+int jacobi_debug_resident(jacobi_t* h, int32_t what);
 
 /* Measurement switch for the halo share of a step (the share of step time
  * that exchanging halos between blocks costs): with on = 1 every block stores

@@ -133,6 +133,7 @@ _SIGS = {
     "jacobi_set_shape": (ctypes.c_int, [P, c_int64, c_int32, P]),
     "jacobi_read_face": (ctypes.c_int, [P, c_int64, c_int32, P, P]),
     "jacobi_debug_drop_block": (ctypes.c_int, [P, c_int64]),
+    "jacobi_debug_resident": (ctypes.c_int, [P, c_int32]),
     "jacobi_measure_local_halo": (ctypes.c_int, [P, c_int32]),
     "jacobi_selftest_dadd": (ctypes.c_int, [P, P, c_int64, P, P]),
     "jacobi_selftest_widen": (ctypes.c_int, [P, P]),
@@ -385,6 +386,10 @@ def jacobi_measure_local_halo(h, on):
 
 def jacobi_debug_drop_block(h, block):
     _call("jacobi_debug_drop_block", h, block)
+
+
+def jacobi_debug_resident(h, what):
+    _call("jacobi_debug_resident", h, what)
 
 
 JACOBI_NOALLOC_MAX_PLANES = 16384

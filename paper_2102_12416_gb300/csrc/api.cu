@@ -671,14 +671,27 @@ StepLaunch step_args(jacobi_t* h, int64_t it, bool all_items) {
 int check_err_word(jacobi_t* h, cudaStream_t s) {
   JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
   JGB_CUDA(cudaStreamSynchronize(s));
+  h->res.unchecked = false;
   if (*h->h_err != DEV_OK) {
     const uint32_t e = *h->h_err;
     JGB_CUDA(cudaMemsetAsync(h->d_err, 0, sizeof(uint32_t), s));
     JGB_CUDA(cudaStreamSynchronize(s));
     return set_error(e == DEV_TIMEOUT ? JACOBI_ETIMEDOUT : JACOBI_ESEQ,
-                     "device-side wait failed (code %u) in the persistent step", e);
+                     "device-side wait failed (code %u) in a persistent or resident step", e);
   }
   return JACOBI_OK;
+}
+
+// Synchronise; after resident launches that nothing has looked at since, the error
+// word comes behind the same wait: they may have given up and left the state as it
+// was, on paths whose other kernels never wait.
+int sync_and_check(jacobi_t* h, cudaStream_t s, bool with_err = false) {
+  with_err = with_err || h->res.unchecked;
+  if (with_err) JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
+  JGB_CUDA(cudaStreamSynchronize(s));
+  if (!with_err) return JACOBI_OK;
+  h->res.unchecked = false;
+  return *h->h_err == DEV_OK ? JACOBI_OK : check_err_word(h, s);  // reads it again, clears it and reports
 }
 
 int step_fused_direct(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
@@ -987,6 +1000,8 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   a.smem = R.smem;
   a.dtype = h->plan.dtype;
   a.emu = h->fp64_emu;
+  a.mute = h->res.debug;
+  if (h->res.debug == kResRefused) a.smem = 2 * kResSmem;  // (test support: more than the device has)
   // A launch holds every SM until it ends: long calls are split, at some 30 to 150
   // ms each, so that other streams get their turn.
   for (int64_t done = 0; done < n;) {
@@ -1002,6 +1017,7 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
     }
     JGB_CUDA(e);
     h->res.launches += 1;
+    h->res.unchecked = true;
     done += a.n_iters;
   }
   return JACOBI_OK;
@@ -1072,14 +1088,10 @@ int compute_bnorm(jacobi_t* h, cudaStream_t s, bool new_state) {
   return JACOBI_OK;
 }
 
-// The norms of every grid to the host; with_err also the error word, behind the
-// same synchronisation.
+// The norms of every grid to the host; with_err also the error word.
 int read_norms(jacobi_t* h, cudaStream_t s, bool with_err = false) {
   JGB_CUDA(cudaMemcpyAsync(h->h_norms, h->d_norms, h->plan.grids.size() * sizeof(GridNorm), cudaMemcpyDeviceToHost, s));
-  if (with_err) JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  JGB_CUDA(cudaStreamSynchronize(s));
-  if (with_err && *h->h_err != DEV_OK) return check_err_word(h, s);  // reads it again, clears it and reports
-  return JACOBI_OK;
+  return sync_and_check(h, s, with_err);
 }
 
 // Host-transfer staging buffer: sized once for the largest padded grid of the
@@ -1662,7 +1674,7 @@ int jacobi_step_timed(jacobi_t* h, int64_t n_iters, void* stream, double* comput
     float a = 0.f;
     if (!rc) cudaEventElapsedTime(&a, ev[0], ev[1]);
     comp = a;
-    if (!rc && (h->path == JACOBI_PATH_PERSISTENT || h->res.ok)) rc = check_err_word(h, s);
+    if (!rc && (h->path == JACOBI_PATH_PERSISTENT || h->res.unchecked)) rc = check_err_word(h, s);
   }
   destroy();
   if (rc) return rc;
@@ -1708,7 +1720,7 @@ int jacobi_solve(jacobi_t* h, double tol, int64_t max_iters, int64_t check_every
         rc = step_with_residual(h, s);
       }
       if (rc) return rc;
-      rc = read_norms(h, s, h->path == JACOBI_PATH_PERSISTENT || h->res.ok);
+      rc = read_norms(h, s, h->path == JACOBI_PATH_PERSISTENT);
       if (rc) return rc;
       const bool stepped = done_k < max_iters;
       bool any_active = false;
@@ -1796,7 +1808,6 @@ int jacobi_copy_out(jacobi_t* h, int64_t grid, void* dst, int32_t dst_on_device,
     if (rc0) return rc0;
     ddst = tmp;
   }
-  int rc = JACOBI_OK;
   cudaError_t e = cudaSuccess;
   if (layout == JACOBI_LAYOUT_PADDED) e = cudaMemsetAsync(ddst, 0, n, s);
   const int parity = (int)(grid_local_iter(h, grid) & 1);
@@ -1804,9 +1815,8 @@ int jacobi_copy_out(jacobi_t* h, int64_t grid, void* dst, int32_t dst_on_device,
     e = launch_gather(h->d_blocks, h->d_geom, (int32_t)G.block_begin, (int32_t)(G.block_end - G.block_begin), G.max_rows, ddst,
                       G.dims.nx, G.dims.ny, parity, layout == JACOBI_LAYOUT_PADDED, h->plan.dtype, s);
   if (e == cudaSuccess && tmp) e = cudaMemcpyAsync(dst, tmp, n, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess && tmp) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) rc = set_error(JACOBI_ECUDA, "copy_out failed: %s", cudaGetErrorString(e));
-  return rc;
+  if (e != cudaSuccess) return set_error(JACOBI_ECUDA, "copy_out failed: %s", cudaGetErrorString(e));
+  return tmp ? sync_and_check(h, s) : JACOBI_OK;
 }
 
 int jacobi_selftest_widen(uint64_t* mismatches, void* stream) {
@@ -1899,8 +1909,7 @@ int jacobi_read_face(jacobi_t* h, int64_t block, int32_t face, void* dst, void* 
   const int64_t height = face < 4 ? B.extent[2] : B.extent[1];
   JGB_CUDA(cudaMemcpy2DAsync(dst, width * e, h->ws + B.recv_off[face][parity], pitch * e, width * e, height,
                              cudaMemcpyDeviceToHost, S(stream)));
-  JGB_CUDA(cudaStreamSynchronize(S(stream)));
-  return JACOBI_OK;
+  return sync_and_check(h, S(stream));
 }
 
 int jacobi_measure_local_halo(jacobi_t* h, int32_t on) {
@@ -1922,6 +1931,12 @@ int jacobi_debug_drop_block(jacobi_t* h, int64_t block) {
   if (!h || block < -1 || block >= (int64_t)h->plan.blocks.size()) return set_error(JACOBI_EINVAL, "bad block");
   h->drop_block = block;
   h->tables_dirty = true;
+  return JACOBI_OK;
+}
+
+int jacobi_debug_resident(jacobi_t* h, int32_t what) {
+  if (!h || what < kResRefused) return set_error(JACOBI_EINVAL, "bad arguments to jacobi_debug_resident");
+  h->res.debug = what;
   return JACOBI_OK;
 }
 

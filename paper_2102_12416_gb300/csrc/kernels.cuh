@@ -228,6 +228,7 @@ struct ResLaunch {
   uint64_t wait_ns;
   int64_t it0, n_iters;
   int32_t n_boxes, smem, dtype, emu;
+  int32_t mute;           // this box sends nothing (test support; < 0: none)
 };
 cudaError_t launch_resident(const ResLaunch& a, cudaStream_t s);
 

@@ -273,13 +273,14 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
     }
     // The sweep's order: shell vectors from the front, the others behind them.
     // Each warp takes 32 consecutive vectors and keeps their order.
+    const int sent = (int)blockIdx.x == a.mute ? 0 : X.faces;
     for (int pass = 0; pass < 2; ++pass) {
       for (int vb = tid & ~31; vb < G.nv; vb += NT) {
         const int v = vb + (tid & 31), row = v / G.nvx, tx = v - row * G.nvx, k = row / G.ny, j = row - k * G.ny;
         bool shell = false;
         if (v < G.nv)
-          shell = (tx == 0 && (X.faces >> XM & 1)) || (tx == G.nvx - 1 && (X.faces >> XP & 1)) || (j == 0 && (X.faces >> YM & 1)) ||
-                  (j == G.ny - 1 && (X.faces >> YP & 1)) || (k == 0 && (X.faces >> ZM & 1)) || (k == G.nz - 1 && (X.faces >> ZP & 1));
+          shell = (tx == 0 && (sent >> XM & 1)) || (tx == G.nvx - 1 && (sent >> XP & 1)) || (j == 0 && (sent >> YM & 1)) ||
+                  (j == G.ny - 1 && (sent >> YP & 1)) || (k == 0 && (sent >> ZM & 1)) || (k == G.nz - 1 && (sent >> ZP & 1));
         const bool mine = v < G.nv && shell == (pass == 0);
         const uint32_t m = __ballot_sync(0xffffffffu, mine);
         int at = 0;

@@ -117,12 +117,15 @@ namespace jgb {
 // lists: behind a workspace of the library's own, or in memory of their own
 // beside a caller's or when a subset of the grids needs more than all did (its
 // boxes are smaller and more).
+constexpr int32_t kResRefused = -2;
 struct Resident {
   bool allowed = true;   // off when the environment asks for a given persistent kernel
   bool ok = false;       // the active grids fit
   int n_boxes = 0, smem = 0;
   int64_t min_iters = 0; // shortest call it takes
   int64_t launches = 0;  // so far, for jacobi_info
+  bool unchecked = false;  // launched since the error word was last looked at
+  int32_t debug = -1;    // jacobi_debug_resident
   char* with_ws = nullptr;
   char* own = nullptr;
   size_t own_bytes = 0;
