@@ -972,7 +972,8 @@ int step_exchange(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s, cudaEvent
 }
 
 // The resident kernel takes calls of res.min_iters iterations or more on the
-// GRAPH and PERSISTENT paths when the active grids fit.  Not under stream
+// GRAPH and PERSISTENT paths when the active grids fit (and no channel is open on
+// the device, see ChannelGate).  Not under stream
 // capture (the cooperative launch would have to be marked in the caller's
 // graph), nor with an injected fault or redirected faces, which are about the
 // other kernels' exchange.
@@ -1032,9 +1033,15 @@ int do_step(jacobi_t* h, int64_t n, cudaStream_t s) {
     return JACOBI_OK;
   }
   if (resident_applies(h, n, s)) {
-    rc = step_resident(h, h->iter, n, s);
-    if (rc == JACOBI_OK) h->iter += n;
-    if (rc != JACOBI_EAGAIN) return rc;
+    int dev = 0;
+    JGB_CUDA(cudaGetDevice(&dev));
+    ChannelGate& gate = channel_gate(dev);
+    std::shared_lock<std::shared_mutex> lock(gate.m);
+    if (gate.open == 0) {
+      rc = step_resident(h, h->iter, n, s);
+      if (rc == JACOBI_OK) h->iter += n;
+      if (rc != JACOBI_EAGAIN) return rc;
+    }
   }
   switch (h->path) {
     case JACOBI_PATH_FUSED: rc = step_fused_direct(h, h->iter, n, s); break;

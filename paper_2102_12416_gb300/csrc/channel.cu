@@ -75,7 +75,17 @@ struct channel_s {
   void* hstage[2] = {nullptr, nullptr};  // pinned host staging of the host-staged form, per receiver
   std::deque<MsgMeta> mailbox[2];        // metadata messages waiting at endpoint e
   uint64_t msg_seq[2] = {0, 0};
+  int dev = -1;            // counted in this device's gate
 };
+
+namespace jgb {
+
+ChannelGate& channel_gate(int dev) {
+  static ChannelGate gates[64];
+  return gates[dev & 63];
+}
+
+}  // namespace jgb
 
 namespace {
 
@@ -272,6 +282,12 @@ __global__ void k_bandwidth(ChanCtr* c, void* slot0, void* slot1, const void* sr
 
 cudaStream_t S(void* s) { return (cudaStream_t)s; }
 
+void gate_count(channel_s* ch, int64_t by) {
+  ChannelGate& g = channel_gate(ch->dev);
+  std::unique_lock<std::shared_mutex> lock(g.m);
+  g.open += by;
+}
+
 int endpoint_of(const channel_s* ch, int64_t block) {
   if (block == ch->block[0]) return 0;
   if (block == ch->block[1]) return 1;
@@ -307,6 +323,10 @@ int channel_open(jacobi_t* h, uint32_t channel_id, int64_t block_a, int64_t bloc
   ch->block[0] = block_a;
   ch->block[1] = block_b;
   ch->max_bytes = max_bytes;
+  if (cudaGetDevice(&ch->dev) != cudaSuccess) {
+    delete ch;
+    return set_error(JACOBI_ECUDA, "no current device");
+  }
   const size_t sb = align_up(max_bytes, 256);
   const size_t total = 4 * sb + 256;
   if (cudaMalloc((void**)&ch->mem, total) != cudaSuccess || cudaMallocHost((void**)&ch->h_err, 64) != cudaSuccess) {
@@ -317,9 +337,11 @@ int channel_open(jacobi_t* h, uint32_t channel_id, int64_t block_a, int64_t bloc
   for (int e = 0; e < 2; ++e)
     for (int p = 0; p < 2; ++p) ch->slot[e][p] = ch->mem + (2 * e + p) * sb;
   ch->ctr = (ChanCtr*)(ch->mem + 4 * sb);
+  gate_count(ch, 1);  // from here on no resident launch is issued; those before it end now
   cudaError_t e = cudaMemset(ch->mem, 0, total);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
+    gate_count(ch, -1);
     cudaFree(ch->mem);
     cudaFreeHost(ch->h_err);
     delete ch;
@@ -523,6 +545,7 @@ int channel_bandwidth(channel_t* ch, size_t bytes, int32_t window, int64_t itera
 int channel_close(channel_t* ch) {
   if (!ch) return JACOBI_OK;
   cudaDeviceSynchronize();
+  gate_count(ch, -1);
   for (int e = 0; e < 2; ++e)
     if (ch->hstage[e]) cudaFreeHost(ch->hstage[e]);
   jacobi_t* h = ch->h;

@@ -6,6 +6,8 @@
 
 #include <cstdarg>
 #include <cstdint>
+#include <mutex>
+#include <shared_mutex>
 #include <string>
 #include <vector>
 
@@ -134,6 +136,18 @@ struct Resident {
   uint32_t* d_ctl = nullptr;
   uint4* d_packets = nullptr;
 };
+
+// Channels open on a device.  A resident launch needs all its SMs at once, while
+// a channel's receive (or a send whose slot is taken) holds SMs until a message of
+// another stream has come: if that message stands behind the launch, neither ends
+// before the wait limit.  So no resident launch is issued while a channel is open:
+// launches hold `m` shared, and channel_open, which takes it alone to count, waits
+// for the device before it hands the channel out.
+struct ChannelGate {
+  std::shared_mutex m;
+  int64_t open = 0;
+};
+ChannelGate& channel_gate(int dev);
 
 }  // namespace jgb
 
