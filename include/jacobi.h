@@ -267,10 +267,13 @@ int jacobi_workspace_bytes_batch(int64_t n_grids, const jacobi_dim3* grids,
 /* Create a solver for one grid.  `init` may be NULL (linear boundary, zero
  * interior).  `workspace` may be NULL (the library allocates and frees it)
  * or a device buffer of at least jacobi_workspace_bytes() bytes, 256-byte
- * aligned, owned by the caller (beside it the library allocates the resident
- * path's tables, a few MB, for grids that path takes, and staging buffers when a
- * call first needs them).  The initial state is written by a kernel on
- * `stream`; the call returns without waiting for it. */
+ * aligned, owned by the caller.  Beside it this call allocates the resident
+ * path's tables, a few MB, for grids which that path takes (nothing with
+ * JACOBI_RESIDENT=0; without memory for them the other kernels run), and calls
+ * that need staging buffers allocate those when they first do; steps and solves
+ * on FUSED, GRAPH and PERSISTENT allocate and free no device memory.  The
+ * initial state is written by a kernel on `stream`; the call returns without
+ * waiting for it. */
 int jacobi_create(jacobi_dim3 grid, jacobi_split split, jacobi_dtype dtype,
                   const jacobi_init* init, void* workspace, size_t ws_bytes, void* stream,
                   jacobi_t** out);

@@ -399,12 +399,15 @@ int plan_build(int64_t n_grids, const jacobi_dim3* grids, const jacobi_split* sp
   P->off_active_blocks = take(nb * sizeof(int32_t));
   P->off_it0 = take(sizeof(int64_t));
   P->off_ticket = take(sizeof(unsigned long long));
-  // Resident path of a handle (the server's requests share step launches).
+  // Resident path of a handle (the server's requests share step launches): room
+  // for the tables of all its grids and of what a solve may leave running, the
+  // first half, quarter and so on of them, whose boxes are smaller and more.
   if (target_items <= 0 && n_grids <= device_sms()) {
     std::vector<ResGrid> rg;
     for (int64_t g = 0; g < n_grids; ++g) rg.push_back(resident_grid(P->grids[g], (int32_t)g));
     ResPlan rp;
-    if (resident_plan(rg, dtype, (int)device_sms(), &rp)) P->res_bytes = resident_layout(rp, rg.size()).bytes;
+    for (; !rg.empty() && resident_plan(rg, dtype, (int)device_sms(), &rp); rg.resize(rg.size() / 2))
+      P->res_bytes = std::max(P->res_bytes, resident_layout(rp, rg.size()).bytes);
   }
   const size_t per16 = 32;  // plane pitch rounded to 32 elements
   for (auto& B : P->blocks) {
@@ -514,38 +517,30 @@ int upload_tables(jacobi_t* h, cudaStream_t s) {
   return JACOBI_OK;
 }
 
-// Boxes and packet buffers of the resident path for the active grids; without
-// them (they do not fit, or there is no memory) the other kernels run.
+// Boxes and packet buffers of the resident path for the active grids, in the
+// memory that the handle has had since its creation: a solve whose grids converge
+// one after another comes here between its checks, where an allocation would stop
+// every stream of the device.  Grids whose tables do not fit are cut into fewer
+// boxes; without a plan or memory the other kernels run.
 int build_resident(jacobi_t* h, cudaStream_t s) {
   Resident& R = h->res;
   R.ok = false;
-  if (!R.allowed || h->plan.res_bytes == 0) return JACOBI_OK;
+  if (!R.allowed || !R.mem) return JACOBI_OK;
   const Plan& P = h->plan;
   std::vector<ResGrid> grids;
   for (int32_t g : h->active_grids) grids.push_back(resident_grid(P.grids[g], g));
   ResPlan rp;
-  if (!resident_plan(grids, P.dtype, (int)device_sms(), &rp) || rp.iter_ns >= rp.launch_ns) return JACOBI_OK;
-  R.min_iters = std::max<int64_t>(4, (int64_t)std::ceil(rp.once_ns / (rp.launch_ns - rp.iter_ns)));
-  const ResLayout L = resident_layout(rp, grids.size());
-  char* mem = R.with_ws;
-  if (!mem || L.bytes > P.res_bytes) {
-    if (L.bytes > R.own_bytes) {
-      if (R.own) cudaFree(R.own);  // (synchronises; the tables are being replaced anyway)
-      R.own = nullptr;
-      R.own_bytes = 0;
-      if (cudaMalloc((void**)&R.own, L.bytes) != cudaSuccess) {
-        cudaGetLastError();
-        R.own = nullptr;
-        return JACOBI_OK;
-      }
-      R.own_bytes = L.bytes;
-    }
-    mem = R.own;
+  ResLayout L{};
+  for (int ctas = (int)device_sms();; ctas = ctas * 3 / 4) {
+    if (!resident_plan(grids, P.dtype, ctas, &rp) || rp.iter_ns >= rp.launch_ns) return JACOBI_OK;
+    L = resident_layout(rp, grids.size());
+    if (L.bytes <= P.res_bytes) break;
   }
-  R.d_boxes = (ResBox*)mem;
-  R.d_grids = (ResGrid*)(mem + L.grids);
-  R.d_ctl = (uint32_t*)(mem + L.ctl);
-  R.d_packets = (uint4*)(mem + L.packets);
+  R.min_iters = std::max<int64_t>(4, (int64_t)std::ceil(rp.once_ns / (rp.launch_ns - rp.iter_ns)));
+  R.d_boxes = (ResBox*)R.mem;
+  R.d_grids = (ResGrid*)(R.mem + L.grids);
+  R.d_ctl = (uint32_t*)(R.mem + L.ctl);
+  R.d_packets = (uint4*)(R.mem + L.packets);
   JGB_CUDA(cudaMemcpyAsync(R.d_boxes, rp.boxes.data(), rp.boxes.size() * sizeof(ResBox), cudaMemcpyHostToDevice, s));
   JGB_CUDA(cudaMemcpyAsync(R.d_grids, grids.data(), grids.size() * sizeof(ResGrid), cudaMemcpyHostToDevice, s));
   JGB_CUDA(cudaMemsetAsync(R.d_ctl, 0, L.bytes - L.ctl, s));  // no packet of the old tables may match a number
@@ -1294,7 +1289,7 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
       return fail(set_error(JACOBI_ENOMEM, "cudaMalloc(%zu) failed: %s", h->plan.bytes, cudaGetErrorString(e)));
     }
     h->own_ws = true;
-    h->res.with_ws = h->ws + ws_end;
+    if (h->plan.res_bytes) h->res.mem = h->ws + ws_end;
   }
   if (cudaMallocHost((void**)&h->h_grids, h->plan.grids.size() * sizeof(GridDev)) != cudaSuccess ||
       cudaMallocHost((void**)&h->h_norms, h->plan.grids.size() * sizeof(GridNorm)) != cudaSuccess ||
@@ -1335,6 +1330,13 @@ int jacobi_create_batch(int64_t n_grids, const jacobi_dim3* grids, const jacobi_
     h->res.allowed = false;  // a persistent kernel was asked for by name
   }
   if (const char* rs = getenv("JACOBI_RESIDENT")) h->res.allowed = atoi(rs) != 0;
+  if (!h->own_ws && h->res.allowed && h->plan.res_bytes) {
+    if (cudaMalloc((void**)&h->res.own, h->plan.res_bytes) != cudaSuccess) {
+      cudaGetLastError();
+      h->res.own = nullptr;
+    }
+    h->res.mem = h->res.own;
+  }
   if (const char* st = getenv("JACOBI_STAGES")) {
     const int v = atoi(st);
     if (v >= 3 && v <= 8) {

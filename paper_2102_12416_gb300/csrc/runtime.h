@@ -115,10 +115,9 @@ void fill_block_tables(const Plan& P, char* ws, int64_t base, int32_t grid_overr
 
 namespace jgb {
 
-// Resident-path tables of one handle (resident.cu), rebuilt with the active
-// lists: behind a workspace of the library's own, or in memory of their own
-// beside a caller's or when a subset of the grids needs more than all did (its
-// boxes are smaller and more).
+// Resident-path tables of one handle (resident.cu), rebuilt with the active lists
+// in memory that it gets at its creation: behind a workspace of the library's own,
+// or an allocation beside a caller's.
 constexpr int32_t kResRefused = -2;
 struct Resident {
   bool allowed = true;   // off when the environment asks for a given persistent kernel
@@ -128,9 +127,8 @@ struct Resident {
   int64_t launches = 0;  // so far, for jacobi_info
   bool unchecked = false;  // launched since the error word was last looked at
   int32_t debug = -1;    // jacobi_debug_resident
-  char* with_ws = nullptr;
-  char* own = nullptr;
-  size_t own_bytes = 0;
+  char* mem = nullptr;   // Plan::res_bytes
+  char* own = nullptr;   // mem, where it is an allocation of its own
   ResBox* d_boxes = nullptr;
   ResGrid* d_grids = nullptr;
   uint32_t* d_ctl = nullptr;
