@@ -320,8 +320,12 @@ int jacobi_set_shape(jacobi_t* h, int64_t zchunk, int32_t cw_cap, void* stream);
  * jacobi_set_shape with a z-chunk of 2, 1, 1/2 or 1/4 times the cost model's
  * and a warp cap of 8, 4, 2 or 0 (tiles; shapes that give the same items are
  * timed once), each on the GRAPH path and the PERSISTENT kernel; then FUSED and the
- * persistent ring depths 3..6 at the best shape.  Applies the fastest (path,
- * ring depth, shape) to `h`.  All candidates give bit-identical iterates.
+ * persistent ring depths 3..6 at the best shape; then, where it takes the
+ * handle's grids, the resident kernel at calls of iters_per_trial iterations
+ * (out->ms_per_iter is its time where those calls run it).  Applies the fastest
+ * (path, ring depth, shape) to `h`; trials shorter than the resident kernel's
+ * calls never choose FUSED for such grids, which would turn it off.  All
+ * candidates give bit-identical iterates.
  * When the environment variable JACOBI_TUNE_CACHE names a file, results are
  * looked up there by a signature of the geometry and appended after a search.
  * Synchronises the stream. */

@@ -1492,13 +1492,17 @@ static int autotune_search(jacobi_t* h, int64_t iters_per_trial, void* stream, j
     int rc = jacobi_create_batch((int64_t)grids.size(), grids.data(), splits.data(), (jacobi_dtype)P.dtype,
                                  inits.data(), nullptr, 0, stream, &t);
     if (rc) return rc;
-    // The candidates are the kernels that path, depth and shape choose between;
-    // calls that the resident kernel takes do not depend on them.
+    // Path, depth and shape choose between the kernels of a launch per iteration
+    // and the persistent ones, which are timed with the resident kernel off.  It
+    // takes calls of res_iters iterations or more on GRAPH and PERSISTENT, and is
+    // timed last, against FUSED, which turns it off.
+    const int64_t res_iters = h->res.allowed && h->res.mem && t->res.ok ? t->res.min_iters : 0;
     t->res.allowed = t->res.ok = false;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    double best = INFINITY;
+    double best = INFINITY, best_other = INFINITY;
+    jacobi_tune_result other{};  // the best that is not FUSED
     // Candidate shapes: the cost model's z-chunk, twice, half and a quarter of
     // it; CTAs of up to 8, 4 or 2 consumer warps (row windows of the
     // corresponding height).  Shapes that plan the same items are tried once.
@@ -1520,17 +1524,17 @@ static int autotune_search(jacobi_t* h, int64_t iters_per_trial, void* stream, j
         seen.push_back(q.items);
         shapes.push_back({zc, cw});
       }
-    // One timed run of n iterations (ms per iteration), after the warm-up.
-    auto timed = [&](int64_t n, double* per) -> int {
+    // A timed run of some calls of n iterations (ms per iteration), after the warm-up.
+    auto timed = [&](int64_t n, double* per, int64_t calls = 1) -> int {
       int rc2 = JACOBI_OK;
       if (cudaEventRecord(e0, s) != cudaSuccess) rc2 = JACOBI_ECUDA;
-      if (!rc2) rc2 = do_step(t, n, s);
+      for (int64_t c = 0; c < calls && !rc2; ++c) rc2 = do_step(t, n, s);
       if (!rc2 && cudaEventRecord(e1, s) != cudaSuccess) rc2 = JACOBI_ECUDA;
       if (!rc2 && cudaEventSynchronize(e1) != cudaSuccess) rc2 = JACOBI_ECUDA;
       if (!rc2) rc2 = check_err_word(t, s);
       float ms = 0.f;
       if (!rc2) cudaEventElapsedTime(&ms, e0, e1);
-      *per = ms / (double)n;
+      *per = ms / (double)(n * calls);
       return rc2;
     };
     // A trial runs at least iters_per_trial iterations and at least ~2 ms (a
@@ -1564,6 +1568,15 @@ static int autotune_search(jacobi_t* h, int64_t iters_per_trial, void* stream, j
         r.cw_cap = cw;
         r.ms_per_iter = per;
       }
+      if (path != JACOBI_PATH_FUSED && per < best_other) {
+        best_other = per;
+        other = r;
+        other.path = path;
+        other.stages = st;
+        other.zchunk = zc;
+        other.cw_cap = cw;
+        other.ms_per_iter = per;
+      }
       return JACOBI_OK;
     };
     // every shape on the graph path and on the persistent kernel (4 stages),
@@ -1581,6 +1594,29 @@ static int autotune_search(jacobi_t* h, int64_t iters_per_trial, void* stream, j
       plan_items(&q, bz, bc, 0, 1);
       if (128 + st * (int64_t)q.max_stage > kMaxStepSmem) continue;
       rc = trial(JACOBI_PATH_PERSISTENT, st, bz, bc);
+    }
+    // The resident kernel at calls of iters_per_trial iterations.  It is what runs
+    // there unless FUSED is chosen; for shorter trials, which it leaves to the other
+    // kernels, FUSED is not, since it would lose the longer calls for good.
+    if (!rc && res_iters > 0 && only_path != JACOBI_PATH_FUSED) {
+      double per = INFINITY;
+      if (iters_per_trial >= res_iters) {
+        t->res.allowed = true;
+        t->path = JACOBI_PATH_GRAPH;
+        t->tables_dirty = true;
+        double est = 0.0;
+        rc = timed(iters_per_trial, &est);
+        const double call_ms = std::max(est, 1e-4) * (double)iters_per_trial;
+        const int64_t calls = std::min<int64_t>(50, std::max<int64_t>(1, (int64_t)std::ceil(2.0 / call_ms)));
+        for (int rep = 0; rep < 2 && !rc; ++rep) {
+          rc = timed(iters_per_trial, &est, calls);
+          per = std::min(per, est);
+        }
+        other.ms_per_iter = per;
+        r.n_tried += 1;
+      }
+      other.n_tried = r.n_tried;
+      if (r.path != JACOBI_PATH_FUSED || iters_per_trial < res_iters || per <= r.ms_per_iter) r = other;
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
