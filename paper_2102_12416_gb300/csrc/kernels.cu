@@ -109,20 +109,20 @@ __device__ __forceinline__ T* ext_row(const BlockDev& B, int p, int j, int k) {
   return (T*)B.u[p] + (int64_t)k * B.plane_pitch + (int64_t)j * B.rx;
 }
 
-// Outside the domain of the integer-pipe adder: sign set, or an exponent field
-// that is too large (FP64) or that of infinities and NaNs (FP32, widened).
+// Outside the domain of the integer-pipe adders: sign set, or an exponent field
+// that is too large.  FP32 states never use them.
 __device__ __forceinline__ bool emu_outside(double v) { return (uint32_t)__double2hiint(v) >= kEmuHiLimit; }
-__device__ __forceinline__ bool emu_outside(float v) { return __float_as_uint(v) >= 0x7F800000u; }
+__device__ __forceinline__ bool emu_outside(float) { return false; }
 
 // A grid whose state holds a value outside that domain is flagged: the step
-// kernels then keep its FP64 sums (the FP64 stencil's, and the FP32 residual's
-// of widened values) on the FP64 pipe.  By the discrete maximum principle
-// Jacobi iterates stay within the range of the boundary and initial data, so a
-// state that passes keeps passing.  The kernels that install a state gather the
-// flag in emu_acc; the |b| reduction that follows them publishes it as emu_bad
-// and clears it for the next state.
+// kernels then keep its sums on the FP64 pipe.  By the discrete maximum
+// principle Jacobi iterates stay within the range of the boundary and initial
+// data, so a state that passes keeps passing.  The kernels that install a state
+// gather the flag in emu_acc; the |b| reduction that follows them publishes it as
+// emu_bad and clears it for the next state.
+template <typename T>
 __device__ __forceinline__ void emu_flag(bool bad, GridNorm* norms, int grid) {
-  if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&norms[grid].emu_acc, 1u);
+  if (sizeof(T) == 8 && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(&norms[grid].emu_acc, 1u);
 }
 
 __device__ __forceinline__ void block_to_shared(BlockDev& d, const BlockDev* s) {
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kThreads) k_init(const BlockDev* __restrict__ 
     const int q = (int)(e < n ? e : e - n), k = q / B.ny, j = q - k * B.ny;
     ((T*)B.recv[e < n ? XM : XP][0])[(int64_t)k * B.ry + j] = value(e < n ? -1 : B.nx, j, k);
   }
-  emu_flag(bad, norms, G.grid);
+  emu_flag<T>(bad, norms, G.grid);
 }
 
 // CTAs [0, n_items) take one work item each and write its |b|^2 partial, straight
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_scatter(const BlockDev* __restr
         }
     }
   }
-  emu_flag(bad, norms, G.grid);
+  emu_flag<T>(bad, norms, G.grid);
 }
 
 // Rows in flight of the gather: a lane holds U rows x E elements.  Rows are kept as

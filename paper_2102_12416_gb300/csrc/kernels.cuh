@@ -221,7 +221,7 @@ struct ResLaunch {
   const ResBox* boxes;
   const ResGrid* rgrids;
   const GridDev* grids;
-  const GridNorm* norms;  // per-grid emu_bad flags
+  const GridNorm* norms;  // per-grid emu_bad flags (FP64 only)
   uint4* packets;
   uint32_t* ctl;          // [0] next sequence number, [1] CTAs that have finished, [2] that have started
   uint32_t* err;
