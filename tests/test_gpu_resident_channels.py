@@ -17,12 +17,13 @@ INIT = dict(bc="uniform", bc_seed=3, interior="zero")
 @pytest.mark.parametrize("zero_copy", [True, False])
 @pytest.mark.parametrize("path", ["graph", "persistent"])
 def test_receive_polls_while_the_step_is_queued(path, zero_copy, own):
-    """Stream a: a step, then the send; stream b: its receive.  Zero-copy it is issued first (one CTA polls), else after the send,
-    which the step keeps back (256 CTAs may poll).  `own`: the channel belongs to the stepping handle, else to another one."""
+    """Stream a: a step, then the send; stream b: its receive.  Zero-copy it is issued first, else after the send, which the step keeps
+    back.  `own`: the channel belongs to the stepping handle, else to another one.  The receive is one CTA: one that polls on every SM
+    (2.4 MB or more) can keep any step out, since an SM divides its memory anew only when it is empty."""
     import paper_2102_12416_gb300 as jg
     u = J.initial_grid(*GRID, dtype=np.float32, **INIT)
     a, b = torch.cuda.Stream(), torch.cuda.Stream()
-    n = 4 << 20
+    n = 16 << 10
     src = torch.arange(n, device="cuda", dtype=torch.int64).to(torch.uint8)
     dst = torch.zeros_like(src)
     torch.cuda.synchronize()
