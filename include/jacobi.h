@@ -140,14 +140,16 @@ typedef struct { int32_t mode; int32_t pad_; int64_t x, y, z; } jacobi_split;
  * the next call that waits for the handle's work (jacobi_sync,
  * jacobi_residual, jacobi_solve, jacobi_step_timed, jacobi_read_face,
  * jacobi_copy_out to the host) returns JACOBI_ETIMEDOUT, and the state is
- * unspecified until jacobi_set_state;
- * state and receive slots of the last iteration are written back.  The launch
- * needs its SMs (up to all of them) at once and holds them to its end.  While a
- * channel is open on the device, whose receives hold SMs until their message has
- * come, it is not used; a kernel of the caller's own that waits for work queued
- * behind a step keeps the step out in the same way.  The environment variable
- * JACOBI_RESIDENT=0 at creation turns it off, as does a set JACOBI_PERSIST_WS; a
- * stream under capture does not use it.
+ * unspecified until jacobi_set_state.  State and receive slots of the last
+ * iteration are written back.  The launch needs its SMs (up to all of them) at
+ * once and holds them to its end; long calls are cut into launches of 2 to 3 ms.
+ * Where handles step on several streams at the same time and would end sooner
+ * sharing the GPU than in turns, the other kernels run.  While a channel is open
+ * on the device, whose receives hold SMs until their message has come, it is not
+ * used; a kernel of the caller's own that waits for work queued behind a step
+ * keeps the step out in the same way.  The environment variable JACOBI_RESIDENT=0
+ * at creation turns it off, as does a set JACOBI_PERSIST_WS; a stream under
+ * capture does not use it.
  * The next three run the halo exchange the way the paper's host-driven
  * runtimes do (Sec. 3, Sec. 4.3), for comparing the exchange forms on the
  * Jacobi3D workload; each iteration is a stencil launch followed by the

@@ -4,6 +4,7 @@
 // runs in the kernels of kernels.cu; this file only plans, uploads tables and
 // launches.
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -546,6 +547,10 @@ int build_resident(jacobi_t* h, cudaStream_t s) {
   JGB_CUDA(cudaMemsetAsync(R.d_ctl, 0, L.bytes - L.ctl, s));  // no packet of the old tables may match a number
   R.n_boxes = (int)rp.boxes.size();
   R.smem = rp.smem;
+  R.iter_ns = rp.iter_ns;
+  R.launch_ns = rp.launch_ns;
+  R.points = 0.0;
+  for (const ResGrid& g : grids) R.points += (double)g.n[0] * g.n[1] * g.n[2];
   R.ok = true;
   return JACOBI_OK;
 }
@@ -663,9 +668,17 @@ StepLaunch step_args(jacobi_t* h, int64_t it, bool all_items) {
   return a;
 }
 
+// Wait for a stream; what the handle had there is over.
+int wait_stream(jacobi_t* h, cudaStream_t s) {
+  JGB_CUDA(cudaStreamSynchronize(s));
+  if (h->note.stream == (void*)s) h->note.until_ns = 0;
+  return JACOBI_OK;
+}
+
 int check_err_word(jacobi_t* h, cudaStream_t s) {
   JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  JGB_CUDA(cudaStreamSynchronize(s));
+  const int rc = wait_stream(h, s);
+  if (rc) return rc;
   h->res.unchecked = false;
   if (*h->h_err != DEV_OK) {
     const uint32_t e = *h->h_err;
@@ -683,8 +696,8 @@ int check_err_word(jacobi_t* h, cudaStream_t s) {
 int sync_and_check(jacobi_t* h, cudaStream_t s, bool with_err = false) {
   with_err = with_err || h->res.unchecked;
   if (with_err) JGB_CUDA(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s));
-  JGB_CUDA(cudaStreamSynchronize(s));
-  if (!with_err) return JACOBI_OK;
+  const int rc = wait_stream(h, s);
+  if (rc || !with_err) return rc;
   h->res.unchecked = false;
   return *h->h_err == DEV_OK ? JACOBI_OK : check_err_word(h, s);  // reads it again, clears it and reports
 }
@@ -980,6 +993,16 @@ bool resident_applies(const jacobi_t* h, int64_t n, cudaStream_t s) {
   return cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
 }
 
+// What the active grids cost by the resident kernel and by the path's other kernels:
+// beside others that keep the GPU busy, a launch per iteration takes its arithmetic
+// (0.0066 and 0.00154 ns a point), a persistent launch 0.0155 and 0.005 (64^3 and
+// 96^3 FP64 and FP32, eight streams).
+StepCost resident_cost(const jacobi_t* h) {
+  const bool f64 = h->plan.dtype == JACOBI_F64;
+  const double pt = h->path == JACOBI_PATH_PERSISTENT ? (f64 ? 0.0155 : 0.005) : (f64 ? 0.0066 : 0.00154);
+  return StepCost{h->res.n_boxes, h->res.iter_ns, h->res.launch_ns, h->res.points * pt};
+}
+
 int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   const Resident& R = h->res;
   ResLaunch a{};
@@ -998,11 +1021,14 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   a.emu = h->fp64_emu;
   a.mute = h->res.debug;
   if (h->res.debug == kResRefused) a.smem = 2 * kResSmem;  // (test support: more than the device has)
-  // A launch holds every SM until it ends: long calls are split, at some 30 to 150
-  // ms each, so that other streams get their turn.
-  for (int64_t done = 0; done < n;) {
+  // A launch holds its SMs until it ends: long calls are split evenly into launches
+  // of 2 to 3 ms (the estimate is up to 1.5 times low), for which other streams'
+  // kernels wait about as long as for a launch of a large grid; a launch's way in
+  // and out, some 14 us, is below 1 % of that.
+  const int64_t parts = (int64_t)std::ceil((double)n * R.iter_ns / 2e6);
+  for (int64_t done = 0, part = 1; done < n; ++part) {
     a.it0 = it0 + done;
-    a.n_iters = std::min<int64_t>(n - done, 16384);
+    a.n_iters = n / parts * part + n % parts * part / parts - done;
     const cudaError_t e = launch_resident(a, s);
     if (e != cudaSuccess && done == 0) {
       // refused before anything ran (say, fewer SMs than the device reports are
@@ -1019,6 +1045,67 @@ int step_resident(jacobi_t* h, int64_t it0, int64_t n, cudaStream_t s) {
   return JACOBI_OK;
 }
 
+struct StepBoard {
+  std::mutex m;
+  std::vector<StepNote*> notes;
+};
+StepBoard& step_board(int dev) {
+  static StepBoard boards[64];
+  return boards[dev & 63];
+}
+
+}  // namespace
+
+namespace jgb {
+
+bool note_steps(int dev, StepNote* me, void* s, int64_t n, const StepCost& cost) {
+  const int64_t now = std::chrono::duration_cast<std::chrono::nanoseconds>(std::chrono::steady_clock::now().time_since_epoch()).count();
+  StepBoard& B = step_board(dev);
+  std::lock_guard<std::mutex> lock(B.m);
+  if (!me->listed) B.notes.push_back(me);
+  me->listed = true;
+  const auto left = [now](const StepNote& o) {  // iterations under way
+    return std::max(0.0, (double)(o.until_ns - now)) / (2.0 * o.per_iter_ns);
+  };
+  // All of them as resident launches one after another, and as others side by side.
+  // Microseconds per iteration of each of 2, 4 and 8 streams on GRAPH, always as
+  // launches, always resident, and by this rule: 32^3 FP32 5.6, 5.9, 6.3; 3.6, 7.2,
+  // 14.5; 3.6, 5.6, 6.1.  64^3 FP64 8.1, 10.1, 18.8; 8.5, 17.0, 34.0; 8.2, 10.1, 19.1.
+  // 96^3 FP32 6.6, 8.0, 15.0; 6.4, 12.8, 25.6; 6.4, 8.0, 14.9.  On PERSISTENT 64^3 FP32
+  // 7.7, 8.3, 9.7; 4.2, 8.4, 16.8; 4.2, 9.1, 9.9, and 96^3 FP64 26, 53, 106; 16, 31, 62;
+  // 16, 31, 62.
+  const double mine = (double)n + left(*me);
+  double turns = mine * cost.iter_ns, longest = mine * cost.launch_ns, busy = mine * cost.share_ns;
+  int boxes = cost.boxes;
+  for (const StepNote* o : B.notes) {
+    if (o == me || o->stream == s) continue;
+    const double it = left(*o);
+    if (it == 0.0) continue;
+    boxes += o->cost.boxes;
+    turns += it * o->cost.iter_ns;
+    longest = std::max(longest, it * o->cost.launch_ns);
+    busy += it * o->cost.share_ns;
+  }
+  // (1.2: iter_ns is low for the smallest grids)
+  const bool take = boxes <= device_sms() || 1.2 * turns <= std::max(longest, busy);
+  const double per = take ? cost.iter_ns : cost.launch_ns;
+  me->stream = s;
+  me->cost = cost;
+  me->per_iter_ns = per;
+  me->until_ns = now + (int64_t)std::min(2.0 * per * mine, 1e18);
+  return take;
+}
+
+void drop_note(int dev, StepNote* me) {
+  StepBoard& B = step_board(dev);
+  std::lock_guard<std::mutex> lock(B.m);
+  B.notes.erase(std::remove(B.notes.begin(), B.notes.end(), me), B.notes.end());
+}
+
+}  // namespace jgb
+
+namespace {
+
 // Advance active grids by n iterations on the selected path.
 int do_step(jacobi_t* h, int64_t n, cudaStream_t s) {
   int rc = refresh_active(h, s);
@@ -1027,10 +1114,8 @@ int do_step(jacobi_t* h, int64_t n, cudaStream_t s) {
     h->iter += std::max<int64_t>(n, 0);
     return JACOBI_OK;
   }
-  if (resident_applies(h, n, s)) {
-    int dev = 0;
-    JGB_CUDA(cudaGetDevice(&dev));
-    ChannelGate& gate = channel_gate(dev);
+  if (resident_applies(h, n, s) && note_steps(h->device, &h->note, s, n, resident_cost(h))) {
+    ChannelGate& gate = channel_gate(h->device);
     std::shared_lock<std::shared_mutex> lock(gate.m);
     if (gate.open == 0) {
       rc = step_resident(h, h->iter, n, s);
@@ -1371,6 +1456,7 @@ int jacobi_create(jacobi_dim3 grid, jacobi_split split, jacobi_dtype dtype, cons
 int jacobi_destroy(jacobi_t* h) {
   if (!h) return JACOBI_OK;
   cudaDeviceSynchronize();
+  drop_note(h->device, &h->note);
   for (channel_s* c : std::vector<channel_s*>(h->channels)) channel_close(c);
   if (h->graph) cudaGraphExecDestroy(h->graph);
   for (auto& pg : h->pgraph)
@@ -1937,7 +2023,6 @@ int jacobi_pipe_rates(double* fp64_adds_per_s, double* int_adds_per_s, void* str
 
 int jacobi_sync(jacobi_t* h, void* stream) {
   if (!h) return set_error(JACOBI_EINVAL, "null handle");
-  JGB_CUDA(cudaStreamSynchronize(S(stream)));
   return check_err_word(h, S(stream));
 }
 

@@ -4,6 +4,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdarg>
 #include <cstdint>
 #include <mutex>
@@ -124,6 +125,8 @@ struct Resident {
   bool ok = false;       // the active grids fit
   int n_boxes = 0, smem = 0;
   int64_t min_iters = 0; // shortest call it takes
+  double iter_ns = 0.0, launch_ns = 0.0;  // estimates (ResPlan)
+  double points = 0.0;   // of the active grids
   int64_t launches = 0;  // so far, for jacobi_info
   bool unchecked = false;  // launched since the error word was last looked at
   int32_t debug = -1;    // jacobi_debug_resident
@@ -146,6 +149,29 @@ struct ChannelGate {
   int64_t open = 0;
 };
 ChannelGate& channel_gate(int dev);
+
+// The steps that the resident kernel could take, one note per handle that has some
+// under way on a device.  Resident launches that do not fit side by side take
+// turns, while launches per iteration of several streams share the GPU: the steps
+// that are under way together are resident or not by which ends them sooner
+// (note_steps).  Times are estimates; a note holds for twice its own, or until its
+// stream has been waited for through the handle.
+struct StepCost {
+  int boxes = 0;
+  double iter_ns = 0.0;    // a resident iteration
+  double launch_ns = 0.0;  // one by the path's other kernels, alone
+  double share_ns = 0.0;   // and with others beside it that keep the GPU busy
+};
+struct StepNote {
+  void* stream = nullptr;
+  std::atomic<int64_t> until_ns{0};
+  double per_iter_ns = 1.0;
+  StepCost cost;
+  bool listed = false;
+};
+// Note n iterations of `me` on stream s; true if they should be resident.
+bool note_steps(int dev, StepNote* me, void* s, int64_t n, const StepCost& cost);
+void drop_note(int dev, StepNote* me);
 
 }  // namespace jgb
 
@@ -198,6 +224,7 @@ struct jacobi_s {
   jgb::GridNorm* h_norms = nullptr;  // pinned, read back from d_norms
   uint32_t* h_err = nullptr;        // pinned
 
+  jgb::StepNote note;             // steps under way that the resident kernel could take
   jgb::Resident res;              // small problems: all iterations of a call on chip
   jgb::KindFork fork;             // side-by-side launch of the step's item kinds
   // CUDA graph of the fused path

@@ -32,7 +32,7 @@ def test_batch_solve_and_long_calls_run_resident():
         assert s.info.resident_launches >= max(iters) // 25  # one between any two checks
     with jg.Jacobi3D((20, 17, 19), ("shape", (8, 8, 8)), "f32", path="graph") as s:
         s.step(20011)
-        assert s.info.resident_launches == 2
+        assert s.info.resident_launches >= 2
 
 
 @pytest.mark.parametrize("env", [{"JACOBI_RESIDENT": "0"}, {"JACOBI_PERSIST_WS": "1"}])
