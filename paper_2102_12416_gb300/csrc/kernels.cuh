@@ -223,6 +223,7 @@ struct ResLaunch {
   const GridDev* grids;
   const GridNorm* norms;  // per-grid emu_bad flags (FP64 only)
   uint4* packets;
+  uint32_t* host_err;     // pinned host word, set beside err
   uint32_t* ctl;          // [0] next sequence number, [1] CTAs that have finished, [2] that have started
   uint32_t* err;
   uint64_t wait_ns;

@@ -394,6 +394,7 @@ __global__ void __launch_bounds__(kResThreads<T>, 1) k_resident(ResLaunch a) {
             }
             if (stop) {
               atomicCAS(a.err, (uint32_t)DEV_OK, (uint32_t)DEV_TIMEOUT);
+              *(volatile uint32_t*)a.host_err = DEV_TIMEOUT;
               ok = false;
               break;
             }

@@ -222,7 +222,7 @@ struct jacobi_s {
   bool tables_dirty = true;
   jgb::GridDev* h_grids = nullptr;   // pinned, uploaded to d_grids
   jgb::GridNorm* h_norms = nullptr;  // pinned, read back from d_norms
-  uint32_t* h_err = nullptr;        // pinned
+  uint32_t* h_err = nullptr;        // pinned: copy of d_err; [1] set by a resident launch that gave up
 
   jgb::StepNote note;             // steps under way that the resident kernel could take
   jgb::Resident res;              // small problems: all iterations of a call on chip
