@@ -412,7 +412,8 @@ int jacobi_read_face(jacobi_t* h, int64_t block, int32_t face, void* dst, void* 
  * bit for bit; other inputs give unspecified values (the step kernels never
  * pass them: a device check keeps such grids on the FP64 pipe).  Setting the
  * environment variable JACOBI_FP64_EMU=0 before jacobi_create keeps every
- * FP64 add of the step kernels on the FP64 pipe.  Asynchronous. */
+ * FP64 add of the handle's kernels on the FP64 pipe (jacobi_residual_noalloc has
+ * no handle and is not affected).  Asynchronous. */
 int jacobi_selftest_dadd(const double* a, const double* b, int64_t n, double* out, void* stream);
 
 /* Test support for the FP32 residual's exact binary32 -> binary64 widening on

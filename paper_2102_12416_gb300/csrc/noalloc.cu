@@ -66,7 +66,7 @@ __device__ __forceinline__ double noalloc_r(float xm, float xp, float ym, float 
 // integer-pipe sums, FP32: 2); the boundary sum is taken only at the points
 // that touch the boundary and the planes are split while they alone do not fill
 // the chip.  256^3 FP64: 528 us with both sums in FP64 at every point and one CTA
-// per plane, 238 us so.
+// per plane, 247 us so.
 template <typename T>
 __global__ void __launch_bounds__(kNaThreads) k_noalloc_planes(const T* __restrict__ u, int64_t nx, int64_t ny, int64_t nz,
                                                              int split, double* scratch) {

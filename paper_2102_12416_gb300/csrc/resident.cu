@@ -11,10 +11,10 @@
 // number of its iteration: an 8-byte access is single-copy atomic, so a reader
 // that finds the number has the payload, and no fence, flag or release is needed.
 // What an iteration costs beside its arithmetic is one store -> L2 -> load trip
-// and one CTA barrier.  Per iteration, launch path -> resident: 32^3 5.1 -> 1.7 us
-// (FP32) and 5.7 -> 2.0 (FP64), 64^3 FP64 6.7 -> 4.2, 96^3 FP32 5.6 -> 3.0 and FP64
-// 11.2 -> 7.9, 128^3 FP32 6.4 -> 5.2; a call costs about 14 us once (launch,
-// tables, the state's way in and out).
+// and one CTA barrier.  Per iteration, launch path -> resident: 32^3 4.9 -> 1.8 us
+// (FP32) and 5.6 -> 2.2 (FP64), 64^3 5.3 -> 2.0 and 6.5 -> 4.1, 96^3 5.5 -> 3.1 and
+// 11.1 -> 7.7, 128^3 FP32 6.5 -> 5.0; a call costs 10 to 40 us once (launch, tables,
+// the state's way in and out).
 //
 // Boxes: each active grid is cut into cx * cy * cz near-equal boxes (x cuts on
 // vector boundaries) regardless of its blocks, so box neighbours always face
